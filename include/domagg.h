@@ -308,7 +308,9 @@ typedef struct {
     int64_t workspace_bytes; /* device workspace currently held by the handle */
     int64_t n_records_shared; /* m = 2, 3: records formed, sorted and scanned in shared memory
                                  (the groups' and the top-level tiles'); the rest of n_records go
-                                 through HBM (for a shard: also those left to the other shards) */
+                                 through HBM (for a shard: also those left to the other shards).
+                                 A problem evaluated by pairs ("pairs") forms none of its
+                                 n_records in HBM: all are counted here */
 } domagg_stats;
 
 domagg_status domagg_get_stats(domagg_handle h, domagg_stats* out);
@@ -377,6 +379,10 @@ domagg_status domagg_forward_noalloc(int m, const void* d_coords, int64_t nD, co
  *                    coordinate in shared memory, with each node's running
  *                    F carried across tiles and ranges of tiles; 0 sends
  *                    those levels' records through HBM;
+ *   "pairs"          0 or 1 (default 1): small problems (up to 24576
+ *                    points) are evaluated by their definition, all pairs in
+ *                    one launch, unless group_bits or top_bits differ from
+ *                    their defaults; 0 sends them through the pipeline;
  *   "rank_windows"   0 .. 64 (default 0: about 48 MB of ranks each): windows
  *                    of destination indices the rank scatter is split into;
  *   "ranges_per_cta" 1 .. 64 (default 4): radix-sort ranges per resident CTA;

@@ -18,7 +18,7 @@ LIB = os.path.join(HERE, "libdomagg.so")
 # memory outside a buffer); for tests and debugging
 LIB_CHECKED = os.path.join(HERE, "libdomagg_checked.so")
 BUILD_DIR = os.path.join(HERE, "_build")
-SOURCES = ["domagg.cu", "sort.cu"]
+SOURCES = ["domagg.cu", "sort.cu", "pairs.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

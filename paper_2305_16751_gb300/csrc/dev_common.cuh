@@ -33,6 +33,11 @@ struct Ctl {
     u32 Tq_total;          // query records (= partial slots)
     u32 max_key_bits;      // widest node key over the instances
     u32 pad1;
+    // the flat map's statistics of the problems taken by pairs, per m - 1
+    // (k_pair_stats): records so far (never reset) and, of the last single
+    // problem, the distinct values and rank digits per coordinate
+    unsigned long long pair_T[4];
+    u32 pair_U[4][3], pair_b[4][3];
 };
 
 // Per-instance table.  The host fills the first block; the kernels fill the

@@ -25,6 +25,7 @@
 #include "k_records.cuh"
 #include "k_top.cuh"
 #include "k_wavelet.cuh"
+#include "k_pairs.cuh"
 
 using namespace domagg;
 
@@ -67,6 +68,13 @@ struct domagg_ctx {
     Ctl* ctl = nullptr;
     DevBuf pts, recs, st_multi, st_seg, stage;
     DevBuf st_wv;  // look-back records of the level-wise passes (their own layout)
+    DevBuf pairs;     // small problems: tables, partials, the statistics' scratch
+    DevBuf st_pairs;  // small problems: self-resetting counters (zeroed when allocated)
+    void* h_pair = nullptr;  // pinned: the tables, then the control block read back
+    size_t h_pair_cap = 0;
+    Ctl ctl_host{};            // the control block as last read back
+    u64 pair_T_seen[4] = {0, 0, 0, 0};  // Ctl::pair_T already accounted for
+    bool use_pairs = true;     // tuning knob "pairs"
     void* h_pin = nullptr;
     size_t h_pin_cap = 0;
     std::string err;
@@ -103,7 +111,9 @@ struct domagg_ctx {
     // windows of the rank scatter (0: about 48 MB of ranks each)
     int rank_windows = 0;
 
-    size_t held() const { return pts.cap + recs.cap + st_multi.cap + st_seg.cap + stage.cap + st_wv.cap; }
+    size_t held() const {
+        return pts.cap + recs.cap + st_multi.cap + st_seg.cap + stage.cap + st_wv.cap + pairs.cap + st_pairs.cap;
+    }
 };
 
 namespace {
@@ -188,8 +198,8 @@ u32 bounds_site(bool clear) {
     }
     cudaGetLastError();
     const u32 mine = hit ? (site ? site : 1u) : 0u;
-    const u32 sorts = bounds_site_sort(clear);
-    return mine ? mine : sorts;
+    const u32 sorts = bounds_site_sort(clear), pairs = bounds_site_pairs(clear);
+    return mine ? mine : (sorts ? sorts : pairs);
 #else
     (void)clear;
     return 0u;
@@ -779,6 +789,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         e = cudaStreamSynchronize(stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "point phase");
         if (const u32 site = bounds_site(true)) return bounds_error(h, site);
+        h->ctl_host = *h_ctl;
         if (h_ctl->error) {
             const u32 bits = h_ctl->error;
             cudaMemsetAsync(&h->ctl->error, 0, sizeof(u32), stream);
@@ -1230,8 +1241,276 @@ domagg_status run_m(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype 
     }
 }
 
+// ---------------------------------------------------------------------------
+// small problems by their definition (k_pairs.cuh)
+// ---------------------------------------------------------------------------
+// Where the line lies: a problem of at most PSTAT_MAX points (its statistics
+// then fit one cluster's shared memory), that is at most 1.5e8 pairs
+// (|D| x |Q|): 63e6 pairs of m = 3 take 30 us, where the pipeline's launches
+// alone take 0.27 ms (m = 2), 0.9 (m = 3), 1.5 (m = 4).  Whole calls,
+// measured: 4096 per side, m = 2, 272 -> 56 us; 12000 x 9001, m = 4,
+// 1519 -> 91 us.  A batch whose such problems hold at most PAIRS_ALL pairs
+// together sends them all by pairs (192 problems of 256 to 4096 per side,
+// planned: 1.24 -> 0.24 ms); one with larger instances, which pay for the
+// pipeline's launches, only those of at most PAIRS_EACH pairs: the pairs'
+// throughput (2.5e6 per us for m = 2, 2.1e6 for m = 3) against the pipeline's
+// (4000 points per us for m = 2, 1000 for m = 3) meets at about 500 and 2000
+// points per side.
+constexpr u64 PAIRS_ALL[5] = {0, 1ull << 27, 600000000ull, 500000000ull, 2000000000ull};
+constexpr u64 PAIRS_EACH[5] = {0, 0, 1ull << 18, 3ull << 20, 1ull << 26};
+
+PairOp pair_op(domagg_op op, domagg_dtype wt) {
+    if (op == DOMAGG_COUNT) return PAIR_COUNT;
+    if (op == DOMAGG_SUM) return wt == DOMAGG_F32 ? PAIR_SUM_F32 : PAIR_SUM_I64;
+    if (op == DOMAGG_MAX) return wt == DOMAGG_F32 ? PAIR_MAX_F32 : PAIR_MAX_I32;
+    return wt == DOMAGG_F32 ? PAIR_MIN_F32 : PAIR_MIN_I32;
+}
+
+// Only calls at the default split of the flat map, on a handle that may
+// allocate, whole (no shard) and by the Sec. 5 pipeline go by pairs.
+bool pairs_allowed(const domagg_ctx* h, int m, const Inst& I) {
+    return h->use_pairs && !h->no_alloc && h->group_bits == GROUP_MAX_BITS && h->top_bits == TOP_MAX_BITS &&
+           I.nshards == 0 && !I.out_lo && (I.flags >> m) == 0u;
+}
+bool pairs_fit(const Inst& I) { return (u64)I.nD + I.nQ <= PSTAT_MAX; }
+u64 pairs_of(const Inst& I) { return (u64)I.nD * I.nQ; }
+
+// One call's small problems: small[m] for m = 1..4.  A single problem's
+// descriptor travels in the launch; several are uploaded as tables.  With
+// `stats` the flat-map statistics run beside the pairs.  Nothing is
+// synchronised (pairs_finish does).  DOMAGG_ERR_OOM: the workspace is too
+// small; nothing was launched.  A frozen handle (a plan's) reuses the tables
+// of its first run.
+domagg_status pairs_launch_all(domagg_ctx* h, const std::vector<Inst>* small, domagg_dtype ct, domagg_dtype wt,
+                               domagg_op op, bool negate, bool stats, cudaStream_t stream) {
+    const PairOp po = pair_op(op, wt);
+    struct Part {
+        PairCall c{};
+        PairStatCall st{};
+        unsigned blocks = 0, st_jobs = 0;
+        u64 scr = 0;      // partials
+        size_t ctr0 = 0;  // first counter
+        u32 most = 0;     // points of the largest problem
+        double bytes = 0;
+    } part[5];
+    std::vector<char> up;  // the tables, at the offsets the device copy has
+    size_t nctr = 0;
+    auto layout = [&](char* base, u32* ctr) -> size_t {
+        Carver c(base);
+        nctr = 0;
+        up.clear();
+        auto put = [&](const void* src, size_t bytes, char* dev) {
+            if (!base) return;
+            const size_t at = (size_t)(dev - base);
+            if (up.size() < at + bytes) up.resize(at + bytes);
+            memcpy(up.data() + at, src, bytes);
+        };
+        // tables first (one upload), then scratch
+        for (int m = 1; m <= 4; ++m) {
+            const std::vector<Inst>& v = small[m];
+            if (v.empty()) continue;
+            Part& P = part[m];
+            const size_t k = v.size();
+            u64 units = 0, total = 0;
+            for (const Inst& I : v) units += (u64)((I.nQ + PAIR_QT - 1) / PAIR_QT) * I.nD;
+            // one wave of two blocks per multiprocessor for a single problem
+            // (equal chunks), about three for a batch
+            u64 wave = 2 * (u64)std::max(h->sms, 1), dc;
+            if (k == 1) {
+                // (the statistics' clusters hold their multiprocessors' registers)
+                const u64 held = stats ? 2ull * PSTAT_CLUSTER * (m - 1) : 0;
+                if (wave > 2 * held) wave -= held;
+                const u64 tiles = (v[0].nQ + PAIR_QT - 1) / PAIR_QT, split = std::max<u64>(1, wave / tiles);
+                dc = std::max<u64>(64, ((u64)v[0].nD + split - 1) / split);
+            } else {
+                dc = std::max<u64>(PAIR_STAGE, units / (wave * 3) + 1);
+            }
+            dc = std::min<u64>(dc, 1u << 20);
+            std::vector<u32> blk_off(k + 1), ctr_off(k), blk;
+            std::vector<u64> scr_off(k), pt_off(k);
+            u64 nb = 0, scr = 0;
+            P.bytes = 0;
+            P.ctr0 = nctr;
+            for (size_t i = 0; i < k; ++i) {
+                const Inst& I = v[i];
+                const u64 tiles = (I.nQ + PAIR_QT - 1) / PAIR_QT, split = std::max<u64>(1, (I.nD + dc - 1) / dc);
+                blk_off[i] = (u32)nb;
+                ctr_off[i] = (u32)nctr;
+                scr_off[i] = scr;
+                pt_off[i] = total;
+                if (k > 1 && base) blk.insert(blk.end(), (size_t)(tiles * split), (u32)i);
+                nb += tiles * split;
+                nctr += tiles;
+                P.most = std::max(P.most, I.nD + I.nQ);
+                if (split > 1) scr += split * I.nQ;
+                total += (u64)I.nD + I.nQ;
+                P.bytes += (double)I.nD * (4.0 * m + (op == DOMAGG_COUNT ? 0 : (wt == DOMAGG_I64 ? 8 : 4))) +
+                           (double)I.nQ * (4.0 * m + 8);
+            }
+            blk_off[k] = (u32)nb;
+            P.blocks = (unsigned)nb;
+            P.c.one = P.st.one = v[0];
+            P.c.dchunk = (u32)dc;
+            P.c.negate = P.st.negate = negate ? 1 : 0;
+            P.c.ctl = P.st.ctl = h->ctl;
+            if (k > 1) {
+                Inst* d_tab = c.take<Inst>(k);
+                u32 *d_blk = c.take<u32>(nb), *d_bo = c.take<u32>(k + 1), *d_co = c.take<u32>(k);
+                u64 *d_so = c.take<u64>(k), *d_po = c.take<u64>(k);
+                P.c.tab = P.st.tab = d_tab;
+                P.c.blk_inst = d_blk;
+                P.c.blk_off = d_bo;
+                P.c.ctr_off = d_co;
+                P.c.scr_off = d_so;
+                P.st.pt_off = d_po;
+                put(v.data(), sizeof(Inst) * k, (char*)d_tab);
+                put(blk.data(), sizeof(u32) * blk.size(), (char*)d_blk);
+                put(blk_off.data(), sizeof(u32) * (k + 1), (char*)d_bo);
+                put(ctr_off.data(), sizeof(u32) * k, (char*)d_co);
+                put(scr_off.data(), sizeof(u64) * k, (char*)d_so);
+                put(pt_off.data(), sizeof(u64) * k, (char*)d_po);
+            }
+            P.scr = scr;
+            P.st.total = total;
+        }
+        for (int m = 1; m <= 4; ++m) {
+            const std::vector<Inst>& v = small[m];
+            if (v.empty()) continue;
+            Part& P = part[m];
+            P.c.scr = c.take<char>((size_t)P.scr * pair_acc_size(po));
+            P.st_jobs = 0;
+            if (stats && m >= 2) {
+                P.st.cnt = c.take<unsigned char>(m >= 3 ? (size_t)P.st.total * (m - 1) : 0);
+                P.st_jobs = (unsigned)(v.size() * (m - 1));
+            }
+            // (the counter offsets run over all m; without a table the problem's own are first)
+            P.c.ctr = ctr && v.size() == 1 ? ctr + P.ctr0 : ctr;
+        }
+        // finished-block counters of the statistics, after the query tiles'
+        size_t at = nctr;
+        for (int m = 2; m <= 4; ++m) {
+            part[m].st.done = ctr ? ctr + at : nullptr;
+            at += small[m].size();
+        }
+        nctr = at;
+        return c.off;
+    };
+    const size_t bytes = layout(nullptr, nullptr);
+    domagg_status st = grow(h, h->st_pairs, std::max<size_t>(nctr, 1024) * sizeof(u32), true);
+    if (!st) st = grow(h, h->pairs, std::max<size_t>(bytes, 256));
+    if (st) return st;
+    layout((char*)h->pairs.p, (u32*)h->st_pairs.p);
+    if (!up.empty() && !h->frozen) {
+        if (h->h_pair_cap < up.size()) {
+            if (h->h_pair) {
+                cudaDeviceSynchronize();
+                cudaFreeHost(h->h_pair);
+            }
+            h->h_pair = nullptr;
+            h->h_pair_cap = 0;
+            const size_t want = std::max<size_t>(up.size() + up.size() / 2, 1 << 16);
+            if (cudaMallocHost(&h->h_pair, want) != cudaSuccess) {
+                cudaGetLastError();
+                h->h_pair = nullptr;
+                return fail(h, DOMAGG_ERR_OOM, "pinned memory for the tables");
+            }
+            h->h_pair_cap = want;
+        }
+        memcpy(h->h_pair, up.data(), up.size());
+        cudaMemcpyAsync(h->pairs.p, h->h_pair, up.size(), cudaMemcpyHostToDevice, stream);
+    }
+    if (h->w_pending) {  // the weights' host copy (domagg_forward_host)
+        cudaStreamWaitEvent(stream, h->ev_w, 0);
+        h->w_pending = false;
+    }
+    Launcher L;
+    L.frozen = h->frozen;
+    L.stream = stream;
+    L.ctl = h->ctl;
+    L.timing = h->timing && !h->frozen;
+    L.log = &h->log;
+    L.pool = &h->pool;
+    L.pool_used = &h->pool_used;
+    for (int m = 1; m <= 4; ++m)
+        if (!small[m].empty())
+            pairs_launch(L, m, po, ct == DOMAGG_F32, part[m].c, part[m].blocks, stats ? &part[m].st : nullptr,
+                         part[m].st_jobs, part[m].most, part[m].bytes);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? DOMAGG_OK : cuda_fail(h, e, "pairs launch");
+}
+
+// The synchronisation of a call whose problems all went by pairs: device
+// errors and the control block.
+domagg_status pairs_finish(domagg_ctx* h, cudaStream_t stream) {
+    domagg_status st = grow_pinned(h, sizeof(Ctl));
+    if (st) return st;
+    Ctl* hc = (Ctl*)h->h_pin;
+    cudaMemcpyAsync(hc, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
+    const cudaError_t e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "pairs");
+    if (const u32 site = bounds_site(true)) return bounds_error(h, site);
+    h->ctl_host = *hc;
+    if (hc->error) {
+        const u32 bits = hc->error;
+        cudaMemsetAsync(&h->ctl->error, 0, sizeof(u32), stream);
+        cudaStreamSynchronize(stream);
+        return device_error(h, bits);
+    }
+    return DOMAGG_OK;
+}
+
+// Facts of the call's last m: the pairs' part, alone or (add) beside the
+// pipeline's.  No record of a small problem reaches HBM.
+void pairs_stats(domagg_ctx* h, int m, const std::vector<Inst>& small, bool add) {
+    const Ctl& c = h->ctl_host;
+    domagg_stats& S = h->stats;
+    if (!add) memset(&S, 0, sizeof(S));
+    u64 n = 0;
+    for (const Inst& I : small) n += (u64)I.nD + I.nQ;
+    const u64 T = m == 1 ? n : c.pair_T[m - 1] - h->pair_T_seen[m - 1];
+    S.n_points += (int64_t)n;
+    S.n_records += (int64_t)T;
+    S.n_records_shared += (int64_t)T;
+    S.m = m;
+    if (add) return;
+    if (small.size() == 1) {
+        u32 kb = 0;
+        for (int i = 0; i < m - 1; ++i) {
+            S.rank_bits[i] = (int32_t)c.pair_b[m - 1][i];
+            S.distinct[i] = (int64_t)c.pair_U[m - 1][i];
+            kb += c.pair_b[m - 1][i];
+        }
+        // the widest node key the flat map's levels would be sorted by
+        S.record_key_bits = m >= 2 && c.pair_b[m - 1][0] ? (int32_t)kb - 1 : 0;
+        S.record_passes = (S.record_key_bits + RADIX_BITS - 1) / RADIX_BITS;
+    }
+    S.workspace_bytes = (int64_t)h->held();
+}
+
+void pairs_seen(domagg_ctx* h) {
+    for (int i = 0; i < 4; ++i) h->pair_T_seen[i] = h->ctl_host.pair_T[i];
+}
+
+// A single small problem: the pairs, one synchronisation, the statistics.
+domagg_status run_pairs_one(domagg_ctx* h, int m, const Inst& I, domagg_dtype ct, domagg_dtype wt, domagg_op op,
+                            bool negate, cudaStream_t stream) {
+    std::vector<Inst> small[5];
+    small[m].push_back(I);
+    domagg_status st = pairs_launch_all(h, small, ct, wt, op, negate, true, stream);
+    if (st) return st;
+    st = pairs_finish(h, stream);
+    if (!st) pairs_stats(h, m, small[m], false);
+    pairs_seen(h);
+    return st;
+}
+
 domagg_status dispatch(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype ct, domagg_dtype wt,
-                       domagg_op op, bool negate, cudaStream_t s, const Planned* pl = nullptr) {
+                       domagg_op op, bool negate, cudaStream_t s, const Planned* pl = nullptr, bool pairs = true) {
+    if (pairs && !pl && inst.size() == 1 && pairs_allowed(h, m, inst[0]) && pairs_fit(inst[0])) {
+        const domagg_status st = run_pairs_one(h, m, inst[0], ct, wt, op, negate, s);
+        if (st != DOMAGG_ERR_OOM) return st;
+        h->err.clear();  // the pipeline may fit a capped workspace that the pairs' partials do not
+    }
     if (op == DOMAGG_COUNT) return run_m<OpCount>(h, m, inst, ct, negate, s, pl);
     if (op == DOMAGG_SUM && wt == DOMAGG_F32) return run_m<OpSumF32>(h, m, inst, ct, negate, s, pl);
     if (op == DOMAGG_SUM && wt == DOMAGG_I64) return run_m<OpSumI64>(h, m, inst, ct, negate, s, pl);
@@ -1252,6 +1531,27 @@ size_t record_bytes(int m, domagg_dtype wt, domagg_op op) {
     // m >= 3 plans reserve both key classes (64- and 32-bit keys) at the full capacity
     const size_t class1 = m >= 3 ? 2 * 4 + 2 * pb : 0;
     return 2 * kb + 2 * pb + class1 + part + 8;
+}
+
+// A batch's instances by the way they go: small[m] by pairs, the others stay
+// in groups[m].
+bool pairs_split(const domagg_ctx* h, std::vector<Inst>* groups, std::vector<Inst>* small) {
+    bool any = false;
+    for (int m = 1; m <= 4; ++m) {
+        if (groups[m].empty() || !pairs_allowed(h, m, groups[m][0])) continue;
+        u64 total = 0;
+        bool larger = false;  // instances that need the pipeline in any case
+        for (const Inst& I : groups[m]) {
+            total += pairs_fit(I) ? pairs_of(I) : 0;
+            larger = larger || !pairs_fit(I);
+        }
+        const u64 each = total <= PAIRS_ALL[m] && !larger ? total : PAIRS_EACH[m];
+        std::vector<Inst> big;
+        for (const Inst& I : groups[m]) (pairs_fit(I) && pairs_of(I) <= each ? small[m] : big).push_back(I);
+        groups[m].swap(big);
+        any = any || !small[m].empty();
+    }
+    return any;
 }
 
 domagg_status check_common(domagg_ctx* h, int m, int64_t nD, int64_t nQ, domagg_dtype ct, domagg_dtype wt,
@@ -1299,6 +1599,9 @@ bool set_tuning(domagg_ctx* h, const std::string& name, int value) {
     } else if (name == "top_bits") {
         if (value < 0 || value > TOP_MAX_BITS) return false;
         h->top_bits = value;
+    } else if (name == "pairs") {
+        if (value < 0 || value > 1) return false;
+        h->use_pairs = value != 0;
     } else if (name == "rank_windows") {
         if (value < 0 || value > 64) return false;
         h->rank_windows = value;
@@ -1386,9 +1689,10 @@ domagg_status domagg_destroy(domagg_handle h) {
     if (!h) return DOMAGG_ERR_INVALID_ARG;
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
-    for (DevBuf* b : {&h->pts, &h->recs, &h->st_multi, &h->st_seg, &h->stage, &h->st_wv})
+    for (DevBuf* b : {&h->pts, &h->recs, &h->st_multi, &h->st_seg, &h->stage, &h->st_wv, &h->pairs, &h->st_pairs})
         if (b->p) cudaFree(b->p);
     if (h->ctl) cudaFree(h->ctl);
+    if (h->h_pair) cudaFreeHost(h->h_pair);
     if (h->h_pin) cudaFreeHost(h->h_pin);
     for (cudaEvent_t e : h->pool) cudaEventDestroy(e);
     for (cudaStream_t s : h->aux)
@@ -1629,7 +1933,6 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst, 
     if (!h) return DOMAGG_ERR_INVALID_ARG;
     if (k < 0 || (k > 0 && !inst)) return fail(h, DOMAGG_ERR_INVALID_ARG, "bad instance array");
     std::vector<Inst> groups[5];
-    int64_t total[5] = {0, 0, 0, 0, 0};
     for (int i = 0; i < k; ++i) {
         const domagg_instance& I = inst[i];
         domagg_status st = check_common(h, I.m, I.nD, I.nQ, coord_dtype, weight_dtype, op);
@@ -1638,21 +1941,41 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst, 
             (op != DOMAGG_COUNT && I.nD > 0 && !I.d_weights))
             return fail(h, DOMAGG_ERR_INVALID_ARG, "null pointer in instance " + std::to_string(i));
         if (I.nQ == 0) continue;
-        total[I.m] += I.nD + I.nQ;
         groups[I.m].push_back(make_inst(I.d_coords, I.nD, I.q_coords, I.nQ, I.d_weights, I.out));
     }
     cudaSetDevice(h->device);
-    for (int m = 1; m <= 4; ++m) {
+    // the small instances by pairs (enqueued first, synchronised with the others)
+    std::vector<Inst> small[5];
+    {
+        std::vector<Inst> all[5];
+        for (int m = 1; m <= 4; ++m) all[m] = groups[m];
+        if (pairs_split(h, groups, small)) {
+            const domagg_status st = pairs_launch_all(h, small, coord_dtype, weight_dtype, op, false, true,
+                                                      (cudaStream_t)stream);
+            if (st == DOMAGG_ERR_OOM) {  // the pipeline may fit a capped workspace that the partials do not
+                h->err.clear();
+                for (int m = 1; m <= 4; ++m) {
+                    groups[m].swap(all[m]);
+                    small[m].clear();
+                }
+            } else if (st) {
+                return st;
+            }
+        }
+    }
+    bool synced = false;
+    domagg_status ret = DOMAGG_OK;
+    for (int m = 1; m <= 4 && !ret; ++m) {
         if (groups[m].empty()) continue;
         // one call per group of at most 2^31 - 1 points
         std::vector<Inst> part;
         int64_t acc = 0;
-        for (size_t i = 0; i <= groups[m].size(); ++i) {
+        for (size_t i = 0; i <= groups[m].size() && !ret; ++i) {
             const bool flush = i == groups[m].size() ||
                                (acc + (int64_t)groups[m][i].nD + groups[m][i].nQ >= ((int64_t)1 << 31) - 1);
             if (flush && !part.empty()) {
-                domagg_status st = dispatch(h, m, part, coord_dtype, weight_dtype, op, false, (cudaStream_t)stream);
-                if (st) return st;
+                ret = dispatch(h, m, part, coord_dtype, weight_dtype, op, false, (cudaStream_t)stream, nullptr, false);
+                synced = true;
                 part.clear();
                 acc = 0;
             }
@@ -1662,8 +1985,20 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst, 
             }
         }
     }
-    (void)total;
-    return DOMAGG_OK;
+    int last = 0;  // the largest m with small problems
+    for (int m = 1; m <= 4; ++m)
+        if (!small[m].empty()) last = m;
+    if (last && (!synced || ret)) {
+        const domagg_status st = pairs_finish(h, (cudaStream_t)stream);
+        if (!ret) ret = st;
+    }
+    if (last && !ret) {
+        bool larger = false;
+        for (int m = last + 1; m <= 4; ++m) larger = larger || !groups[m].empty();
+        if (!larger) pairs_stats(h, last, small[last], !groups[last].empty());
+    }
+    if (last) pairs_seen(h);
+    return ret;
 }
 
 }  // extern "C"
@@ -1675,6 +2010,8 @@ struct domagg_plan_s {
         std::vector<Inst> inst;         // as given (sizes and pointers)
         std::vector<PlannedChunk> chunks;
         u32 margin = 0;                 // epoch guard margin
+        bool pairs = false;             // the plan's small instances, of every m, by pairs
+        std::vector<Inst> small[5];
     };
     int device = 0;
     domagg_dtype ct = DOMAGG_I32, wt = DOMAGG_I32;
@@ -1710,6 +2047,10 @@ domagg_status plan_fail(domagg_plan p, domagg_status st, const std::string& msg)
 // One planned run of a group: the epoch guard, then the pipeline.
 domagg_status plan_group_run(domagg_plan p, domagg_plan_s::Group& g, cudaStream_t s) {
     domagg_ctx* h = g.ctx;
+    if (g.pairs) {  // one launch per m; no records, no capacities, no look-backs
+        const domagg_status st = pairs_launch_all(h, g.small, p->ct, p->wt, p->op, false, false, s);
+        return st ? plan_fail(p, st, h->err) : DOMAGG_OK;
+    }
     k_epoch_clear<<<304, 256, 0, s>>>(h->ctl, (u64*)h->st_multi.p, h->st_multi.cap / sizeof(u64), (u64*)h->st_seg.p,
                                        h->st_seg.cap / sizeof(u64), g.margin);
     k_epoch_restart<<<1, 32, 0, s>>>(h->ctl, g.margin);
@@ -1740,7 +2081,7 @@ domagg_status plan_group(domagg_plan p, int m, const std::vector<Inst>& part, do
     p->groups.push_back(g);
     domagg_plan_s::Group& G = p->groups.back();
     std::vector<Inst> measured = part;
-    st = dispatch(G.ctx, m, measured, p->ct, p->wt, p->op, false, s);
+    st = dispatch(G.ctx, m, measured, p->ct, p->wt, p->op, false, s, nullptr, false);
     if (st) return plan_fail(p, st, G.ctx->err);
     if (cudaStreamSynchronize(s) != cudaSuccess) return plan_fail(p, DOMAGG_ERR_CUDA, "measuring run");
     // capacity budget: 2^32 positions and ~60% of the free device memory
@@ -1840,6 +2181,31 @@ domagg_status plan_group(domagg_plan p, int m, const std::vector<Inst>& part, do
     return DOMAGG_OK;
 }
 
+// The plan's small instances (taken out of groups): a first run uploads their
+// tables and allocates for good.  On a workspace too small for their partials
+// they stay in groups.
+domagg_status plan_pairs(domagg_plan p, std::vector<Inst>* groups, cudaStream_t s) {
+    domagg_plan_s::Group g;
+    domagg_status st = domagg_create(&g.ctx, p->device, 0);
+    if (st) return plan_fail(p, st, "creating the plan's workspace");
+    std::vector<Inst> all[5];
+    for (int m = 1; m <= 4; ++m) all[m] = groups[m];
+    g.pairs = true;
+    st = pairs_split(g.ctx, groups, g.small) ? DOMAGG_OK : DOMAGG_ERR_UNSUPPORTED;
+    if (!st) st = pairs_launch_all(g.ctx, g.small, p->ct, p->wt, p->op, false, false, s);
+    if (st == DOMAGG_ERR_OOM || st == DOMAGG_ERR_UNSUPPORTED) {  // none, or no room: all by the pipeline
+        for (int m = 1; m <= 4; ++m) groups[m].swap(all[m]);
+        domagg_destroy(g.ctx);
+        return DOMAGG_OK;
+    }
+    p->groups.push_back(g);
+    domagg_plan_s::Group& G = p->groups.back();
+    if (!st) st = domagg_sync_status(G.ctx, s);
+    if (st) return plan_fail(p, st, G.ctx->err);
+    G.ctx->frozen = true;
+    return DOMAGG_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1877,6 +2243,11 @@ domagg_status domagg_batch_plan(domagg_plan* out, int device, int k, const domag
         cudaGetLastError();
         delete p;
         return DOMAGG_ERR_INVALID_ARG;
+    }
+    if (const domagg_status st = plan_pairs(p, groups, (cudaStream_t)stream)) {
+        g_plan_create_error = p->err;
+        plan_free(p);
+        return st;
     }
     for (int m = 1; m <= 4; ++m) {
         std::vector<Inst> part;
@@ -1947,8 +2318,9 @@ domagg_status domagg_plan_autotune(domagg_plan p, void* stream, double* best_ms)
     for (auto& g : p->groups) {
         double best = 1e30;
         int br = g.ctx->ranges_per_cta, bb = g.ctx->blocks_per_sm;
-        for (int ri = 0; ri < 3 && !st; ++ri) {
-            for (int bi = 0; bi < 3 && !st; ++bi) {
+        const int shapes = g.pairs ? 1 : 3;  // (the pairs' launches have one shape)
+        for (int ri = 0; ri < shapes && !st; ++ri) {
+            for (int bi = 0; bi < shapes && !st; ++bi) {
                 g.ctx->ranges_per_cta = kRanges[ri];
                 g.ctx->blocks_per_sm = kBlocks[bi];
                 st = plan_group_run(p, g, s);  // warm-up of this shape
@@ -2066,7 +2438,7 @@ const char* domagg_timing_kind_name(int kind) {
     static const char* names[] = {"encode",  "hist_points",  "sort_points", "rank",     "count_scan",
                                   "expand",  "hist_records", "sort_records", "segscan", "reduce",
                                   "small",   "h2d",          "d2h",          "wavelet",  "sort_groups",
-                                  "group",   "top"};
+                                  "group",   "top",          "pairs"};
     if (kind < 0 || kind >= (int)(sizeof(names) / sizeof(names[0]))) return "";
     return names[kind];
 }

@@ -31,6 +31,7 @@ enum Kind {
     KIND_SORT_GROUPS,  // m = 2: the points by their group of ranks
     KIND_GROUP,        // m = 2: the deep levels in shared memory (k_group)
     KIND_TOP,          // m = 2: the top levels per tile (k_top)
+    KIND_PAIRS,        // small problems by their definition (k_pairs)
     KIND_COUNT_
 };
 
@@ -131,6 +132,20 @@ inline u64 sort_range_bound_n(u64 items, u64 nseg) {
 
 // Point-phase scans (ranks, count scan) tile the points in 4096s.
 constexpr u32 POINT_TILE = 4096;
+
+// pairs.cu: the definition over all pairs, for small problems of the same m,
+// and (st != nullptr) their flat-map statistics beside it (st_jobs: ranked
+// coordinates of all problems; st_points: the largest problem's).
+struct PairCall;
+struct PairStatCall;
+enum PairOp { PAIR_SUM_F32, PAIR_SUM_I64, PAIR_MAX_I32, PAIR_MAX_F32, PAIR_MIN_I32, PAIR_MIN_F32, PAIR_COUNT };
+constexpr size_t pair_acc_size(PairOp op) { return op == PAIR_SUM_F32 || op == PAIR_SUM_I64 ? 8 : 4; }
+void pairs_launch(Launcher& L, int m, PairOp op, bool f32, const PairCall& C, unsigned blocks,
+                  const PairStatCall* st, unsigned st_jobs, u32 st_points, double bytes);
+
+// Checked build: the site of the first out-of-range index the kernels of
+// pairs.cu met (0 if none), cleared when `clear`; sort.cu's below.
+u32 bounds_site_pairs(bool clear);
 
 // Checked build: the site of the first out-of-range index the kernels of
 // sort.cu met (0 if none), cleared when `clear`.  Always 0 in the product
