@@ -911,7 +911,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                      (u64*)h->st_multi.p, (double)N, (u32*)P[24], sort_range_bound(pt_sizes),
                      planned ? nullptr : &gb_host, N};
         sort_pairs<u32, u64>(L, gs, gkey, gval, false, gbits_max, 0xffffffffu, KIND_HIST_POINTS, KIND_SORT_GROUPS,
-                             gbits, true, false);
+                             gbits, true);
         L.start(KIND_SMALL, 0.0);
         k_group_slots<<<1, 1024, 0, stream>>>(d_inst, k, gslot);
         L.stop();
@@ -1123,7 +1123,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                          (u64*)h->st_multi.p, (double)C.T0, (u32*)R[10], nrb0, planned ? nullptr : &sbits_host, C.T0};
             const K keymask = ~(K(1) << (sizeof(K) * 8 - 1));  // all but the role bit
             sort_pairs<K, Pay>(L, rs, keys, pays, false, C.key_bits, keymask, KIND_HIST_RECORDS, KIND_SORT_RECORDS,
-                               d_sbits, true, M <= 2);
+                               d_sbits, true);
         }
         if (C.T1 > 0 && npass1 > 0 && nseg1 > 0) {
             std::vector<u32> sbits_host;

@@ -10,6 +10,8 @@
 // digits keep their order) is what lets the pipeline pre-order points by the
 // last coordinate and then sort records by node key only (Sec. 5).
 #pragma once
+#include <type_traits>
+
 #include "dev_common.cuh"
 
 namespace domagg {
@@ -57,29 +59,23 @@ __device__ __forceinline__ TileLoc locate_range(u32 r, const u32* seg_off, const
 
 // Digit histograms of all passes, per segment: hist[(seg*npass + p)*RADIX + d].
 // One block per range of `range_items` items (ranges never straddle a
-// segment); counts are aggregated per warp with match_any before the
-// shared-memory atomics, so skewed digits do not serialise.  With seg_bits,
-// a segment only counts the passes its keys have digits for (the others
-// skip it).  With `uniform` (keys whose digits are spread evenly, as the
-// m <= 2 node keys: a prefix of a dense rank), digits with at least 5
-// significant bits are counted with plain shared atomics.
+// segment), per-warp counts in shared memory.  With seg_bits, a segment only
+// counts the passes its keys have digits for (the others skip it).
 template <typename K>
 __global__ __launch_bounds__(256) void k_radix_hist(const K* __restrict__ keys, const u32* __restrict__ seg_off,
                                                     const u32* __restrict__ range_off, int nseg, u32 range_items,
                                                     int npass, int shift0, K keymask, u32* __restrict__ hist,
-                                                    u32* __restrict__ range_cnt0, const u32* __restrict__ seg_bits,
-                                                    int uniform) {
+                                                    u32* __restrict__ range_cnt0,
+                                                    const u32* __restrict__ seg_bits) {
     extern __shared__ u32 sh_hist[];  // [8 warps][npass][RADIX]
     const u32 r = blockIdx.x;
     if (r >= __ldg(range_off + nseg)) return;
-    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const u32 warp = threadIdx.x >> 5;
     for (int x = threadIdx.x; x < 8 * npass * RADIX; x += 256) sh_hist[x] = 0;
     __syncthreads();
     const TileLoc L = locate_range(r, seg_off, range_off, nseg, range_items);
     const int sbits = seg_bits ? (int)__ldg(seg_bits + L.seg) : 0;
     const int np = seg_bits ? min(npass, (sbits + RADIX_BITS - 1) / RADIX_BITS) : npass;
-    // passes [0, spread) have digits with at least 5 significant bits
-    const int spread = (seg_bits && uniform && sbits >= 5) ? min(np, (sbits - 5) / RADIX_BITS + 1) : 0;
     u32* wh = sh_hist + warp * npass * RADIX;
     for (u32 base = L.start; base < L.end; base += 256u * 8u) {
         K kk[8];
@@ -90,18 +86,9 @@ __global__ __launch_bounds__(256) void k_radix_hist(const K* __restrict__ keys, 
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const bool valid = base + (u32)j * 256u + threadIdx.x < L.end;
-            for (int p = 0; p < np; ++p) {
-                const u32 d = digit_of(kk[j], keymask, shift0 + p * RADIX_BITS);
-                // a digit with at least 5 significant bits of a node key is spread
-                // out: plain shared atomics; otherwise (and for point keys, whose
-                // spread is unknown) lanes sharing lane 0's digit add together
-                if (p < spread) {
-                    if (valid) atomicAdd(wh + p * RADIX + d, 1u);
-                } else {
-                    warp_hist_add(wh + p * RADIX, d, valid, lane);
-                }
-            }
+            if (base + (u32)j * 256u + threadIdx.x < L.end)
+                for (int p = 0; p < np; ++p)
+                    atomicAdd(wh + p * RADIX + digit_of(kk[j], keymask, shift0 + p * RADIX_BITS), 1u);
         }
     }
     __syncthreads();
@@ -114,40 +101,76 @@ __global__ __launch_bounds__(256) void k_radix_hist(const K* __restrict__ keys, 
     }
 }
 
-// First-pass global position of every (range, digit): the digit's start in
-// the segment plus the counts of the segment's earlier ranges.  In place over
-// the per-range counts.  Grid (segment, group of 32 digits); the 32 warps of
-// a block split the segment's ranges into 32 slices (lane = digit): slice
-// sums, an exclusive scan of them in shared memory, then the running bases.
-constexpr int RB_WARPS = 32;
-static __global__ __launch_bounds__(RB_WARPS * 32) void k_range_bases(const u32* __restrict__ range_off,
-                                                                     const u32* __restrict__ digit_off, int npass,
-                                                                     u32* __restrict__ range_cnt0) {
-    __shared__ u32 s_sum[RB_WARPS][33];
+// Digit counts of every range for one pass (the first pass takes them from
+// k_radix_hist): range_cnt[r*RADIX + d].
+template <typename K>
+__global__ __launch_bounds__(256) void k_range_count(const K* __restrict__ keys, const u32* __restrict__ seg_off,
+                                                     const u32* __restrict__ range_off, int nseg, u32 range_items,
+                                                     int shift, K keymask, u32* __restrict__ range_cnt) {
+    __shared__ u32 s_wh[8][RADIX];
+    const u32 r = blockIdx.x;
+    if (r >= __ldg(range_off + nseg)) return;
+    u32* wh = s_wh[threadIdx.x >> 5];
+    for (int x = threadIdx.x; x < 8 * RADIX; x += 256) (&s_wh[0][0])[x] = 0u;
+    __syncthreads();
+    const TileLoc L = locate_range(r, seg_off, range_off, nseg, range_items);
+    for (u32 base = L.start; base < L.end; base += 256u * 8u) {
+        K kk[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const u32 x = base + (u32)j * 256u + threadIdx.x;
+            kk[j] = x < L.end ? keys[x] : K(0);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (base + (u32)j * 256u + threadIdx.x < L.end) atomicAdd(wh + digit_of(kk[j], keymask, shift), 1u);
+    }
+    __syncthreads();
+    u32 c = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) c += s_wh[w][threadIdx.x];
+    range_cnt[(u64)r * RADIX + threadIdx.x] = c;
+}
+
+// Global position of every (range, digit): the digit's start in the segment
+// (digit_off of the pass) plus the counts of the segment's earlier ranges.
+// In place over the per-range counts.  Grid (segment, group of 32 digits);
+// the WARPS warps of a block split the segment's ranges into slices (lane =
+// digit): slice sums, an exclusive scan of them in shared memory, then the
+// running bases.  32 warps for few segments of many ranges, one for many
+// segments of few.
+template <int WARPS>
+__global__ __launch_bounds__(WARPS * 32) void k_range_bases(const u32* __restrict__ range_off,
+                                                            const u32* __restrict__ digit_off, int npass,
+                                                            u32* __restrict__ range_cnt) {
+    __shared__ u32 s_sum[WARPS][33];
     const int seg = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = blockIdx.y * 32 + lane;
     const u32 r0 = __ldg(range_off + seg), r1 = __ldg(range_off + seg + 1);
-    const u32 n = r1 - r0, per = (n + RB_WARPS - 1) / RB_WARPS;
+    const u32 n = r1 - r0, per = (n + WARPS - 1) / WARPS;
+    if (n == 0u) return;
     const u32 a = r0 + min(n, (u32)warp * per), b = r0 + min(n, (u32)(warp + 1) * per);
-    u32 sum = 0;
-    for (u32 r = a; r < b; r += 16) {  // 16 loads in flight
-        u32 c[16];
+    u32 run = __ldg(digit_off + (u64)seg * npass * RADIX + d);
+    if (WARPS > 1) {
+        u32 sum = 0;
+        for (u32 r = a; r < b; r += 16) {  // 16 loads in flight
+            u32 c[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) c[i] = r + i < b ? range_cnt0[(u64)(r + i) * RADIX + d] : 0u;
+            for (int i = 0; i < 16; ++i) c[i] = r + i < b ? range_cnt[(u64)(r + i) * RADIX + d] : 0u;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sum += c[i];
+            for (int i = 0; i < 16; ++i) sum += c[i];
+        }
+        s_sum[warp][lane] = sum;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) run += s_sum[w][lane];
     }
-    s_sum[warp][lane] = sum;
-    __syncthreads();
-    u32 run = __ldg(digit_off + (u64)seg * npass * RADIX + d);  // pass 0
-    for (int w = 0; w < warp; ++w) run += s_sum[w][lane];
     for (u32 r = a; r < b; r += 16) {
         u32 c[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) c[i] = r + i < b ? range_cnt0[(u64)(r + i) * RADIX + d] : 0u;
+        for (int i = 0; i < 16; ++i) c[i] = r + i < b ? range_cnt[(u64)(r + i) * RADIX + d] : 0u;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            if (r + i < b) range_cnt0[(u64)(r + i) * RADIX + d] = run;
+            if (r + i < b) range_cnt[(u64)(r + i) * RADIX + d] = run;
             run += c[i];
         }
     }
@@ -188,22 +211,24 @@ constexpr int ONESWEEP_THREADS = 256;
 #define ONESWEEP_MIN_CTAS 3
 #endif
 
-// Shared-memory layout of the persistent onesweep kernel: two tile buffers
-// (keys, then values, each with 16 bytes of alignment slack at both ends),
-// the warp histograms and the per-digit bases.
-template <typename K, typename V, int TILE>
+// Shared memory: the tile in digit order, the warps' digit counts (then first
+// positions), per digit the global position of tile position 0 and the next
+// global position.
+template <typename K, typename V>
 struct OnesweepSmem {
     static constexpr int WARPS = ONESWEEP_THREADS / 32;
-    static constexpr size_t KBYTES = ((size_t)(TILE + 2 * 16 / sizeof(K)) * sizeof(K) + 15) & ~(size_t)15;
-    static constexpr size_t VBYTES = ((size_t)(TILE + 2 * 16 / sizeof(V)) * sizeof(V) + 15) & ~(size_t)15;
-    static constexpr size_t BUF = KBYTES + VBYTES;
-    static constexpr size_t WHIST = (size_t)WARPS * (RADIX + 1) * 4;
-    static constexpr size_t TOTAL = 2 * BUF + WHIST + 2 * RADIX * 4 + 64;
+    static constexpr int TILE = ONESWEEP_THREADS * onesweep_items<K, V>();
+    static constexpr size_t KEYS = 0;
+    static constexpr size_t VALS = KEYS + (size_t)TILE * sizeof(K);
+    static constexpr size_t WHIST = (VALS + (size_t)TILE * sizeof(V) + 15) & ~(size_t)15;
+    static constexpr size_t GDST = WHIST + (size_t)WARPS * RADIX * 4;
+    static constexpr size_t RUN = GDST + RADIX * 4;
+    static constexpr size_t TOTAL = RUN + RADIX * 4;
 };
 
 template <typename K, typename V>
 __host__ __device__ constexpr size_t onesweep_smem() {
-    return OnesweepSmem<K, V, ONESWEEP_THREADS * onesweep_items<K, V>()>::TOTAL;
+    return OnesweepSmem<K, V>::TOTAL;
 }
 
 // One LSD pass: stable scatter of every segment by digit `pass`.
@@ -214,97 +239,176 @@ __host__ __device__ constexpr size_t onesweep_smem() {
 //   2. publishes the count and runs one decoupled look-back over the earlier
 //      ranges of the segment (bounded waits), which gives the global position
 //      of the range's first item of every digit,
-//   3. streams the range tile by tile: the next tile's keys and values are
-//      fetched into the other shared-memory buffer by TMA bulk copies
-//      (cp.async.bulk, completion on an mbarrier) while the current tile is
-//      ranked (warp-level stable match_any ranking), sorted locally in shared
-//      memory and written out with coalesced stores at running per-digit
-//      positions.
+//   3. takes the range tile by tile: keys and values into registers (warp w
+//      holds consecutive items, coalesced), the rank of every item among its
+//      warp's items of the same digit (8-ballot match), the tile in digit
+//      order through shared memory, and coalesced stores at the running
+//      global position of every digit.
 // There is no inter-CTA wait inside a range; the look-back runs once per
-// range (hundreds of thousands of items), not once per tile.
+// range (tens of thousands of items), not once per tile.
+//
+// Bound by instruction issue, on the half-rate pipe of the digit match above
+// all (110 instructions per item without a look-back), and by the tile's
+// barriers.  Keys and values wait in registers and a tile is staged in shared
+// memory once, in digit order; with the ranges' positions from k_range_count
+// a pass over 6.3e6 pairs of 4 + 4 bytes takes 45 us instead of 69 (with TMA
+// double buffers and the look-back), over 2^25 pairs 0.22 ms instead of 0.28.
+// Three CTAs of 16 items per thread: four spill (64 registers; 2.65 instead
+// of 2.35 ms over the point sorts at 2^25), 12 items move more, shorter runs.
 //
 // IOTA: the values are the items' own global indices (first pass of a sort
 // that returns a permutation); `vin` is not read.
 // STABLE = false (the dense-rank sorts, where only the sorted key sequence
 // matters) ranks with one shared-memory atomic per item instead of the digit
-// match.  range_base (first pass only, may be null) holds every range's
-// global position per digit, which replaces the range's count and look-back.
+// match.  range_base (may be null) holds every range's global position per
+// digit, which replaces the range's count and look-back.
 template <typename K, typename V, bool IOTA, bool STABLE>
 __global__ __launch_bounds__(ONESWEEP_THREADS, ONESWEEP_MIN_CTAS) void k_onesweep(
     const K* __restrict__ kin, const V* __restrict__ vin, K* __restrict__ kout, V* __restrict__ vout,
     const u32* __restrict__ seg_off, const u32* __restrict__ range_off, int nseg, u32 range_items,
     const u32* __restrict__ seg_bits, const u32* __restrict__ range_base, const u32* __restrict__ digit_off,
-    int npass, int pass, int shift, K keymask, u64* status, Ctl* ctl, int launch_idx, int uniform) {
+    int npass, int pass, int shift, K keymask, u64* status, Ctl* ctl, int launch_idx) {
     constexpr int THREADS = ONESWEEP_THREADS, ITEMS = onesweep_items<K, V>();
     constexpr int TILE = THREADS * ITEMS, WARPS = THREADS / 32;
-    typedef OnesweepSmem<K, V, TILE> SM;
-    constexpr u32 KAL = 16 / sizeof(K), VAL = 16 / sizeof(V);  // items per 16 bytes
+    typedef OnesweepSmem<K, V> SM;
+    static_assert(SM::TILE == TILE && THREADS == RADIX && ITEMS % 2 == 0, "one thread per digit");
     extern __shared__ __align__(128) unsigned char smem[];
-    u32* s_whist = reinterpret_cast<u32*>(smem + 2 * SM::BUF);  // [WARPS][RADIX+1]
-    u32* s_dstart = s_whist + WARPS * (RADIX + 1);              // tile-local digit starts
-    u32* s_run = s_dstart + RADIX;                              // next global position per digit
-    u64* s_bar = reinterpret_cast<u64*>(s_run + RADIX);         // [2]
-    u32* s_info = reinterpret_cast<u32*>(s_bar + 2);            // range, koff[2], voff[2], epoch, abort
-
+    K* s_k = reinterpret_cast<K*>(smem + SM::KEYS);
+    V* s_v = reinterpret_cast<V*>(smem + SM::VALS);
+    u32* s_wh = reinterpret_cast<u32*>(smem + SM::WHIST);  // [WARPS][RADIX]
+    u32* s_gdst = reinterpret_cast<u32*>(smem + SM::GDST);
+    u32* s_run = reinterpret_cast<u32*>(smem + SM::RUN);
+    __shared__ u32 s_scan[WARPS];
+    __shared__ u32 s_range;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const u32 nranges = __ldg(range_off + nseg);
     const u32 lt = lanemask_lt();
-    // TMA loads of items [a, e) into buffer b (one thread)
-    auto issue = [&](int b, u32 a, u32 e) {
-        const u32 ka = a / KAL * KAL, kb = (e + KAL - 1) / KAL * KAL;
-        const u32 kbytes = (kb - ka) * (u32)sizeof(K);
-        u32 vbytes = 0, va = 0;
-        if (!IOTA) {
-            va = a / VAL * VAL;
-            const u32 vb = (e + VAL - 1) / VAL * VAL;
-            vbytes = (vb - va) * (u32)sizeof(V);
-        }
-        s_info[1 + b] = a - ka;
-        s_info[3 + b] = a - va;
-        unsigned char* buf = smem + b * SM::BUF;
-        mbar_arrive_expect_tx(&s_bar[b], kbytes + vbytes);
-        bulk_g2s(buf, kin + ka, kbytes, &s_bar[b]);
-        if (!IOTA) bulk_g2s(buf + SM::KBYTES, vin + va, vbytes, &s_bar[b]);
+    const u32 epoch = ctl->epoch_base + (u32)launch_idx;
+    u32* wh = s_wh + warp * RADIX;
+    auto clear_counts = [&]() {  // the warp's own row
+#pragma unroll
+        for (int x = 0; x < RADIX / 32 / 4; ++x)
+            reinterpret_cast<uint4*>(wh)[x * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
     };
-    if (tid == 0) {
-        mbar_init(&s_bar[0], 1);
-        mbar_init(&s_bar[1], 1);
-        fence_mbar_init();
-        s_info[5] = ctl->epoch_base + (u32)launch_idx;
-        s_info[6] = 0;
-    }
-    __syncthreads();
-    const u32 epoch = s_info[5];
-    u32 phase[2] = {0u, 0u};
-    bool pending[2] = {false, false};  // thread 0's view of copies in flight
-    int b = 0;
+
+    // one tile of n items from a (FULL: n == TILE)
+    auto do_tile = [&](auto full, u32 a, u32 n, u32 seg_begin, u32 seg_len) {
+        constexpr bool FULL = decltype(full)::value;
+        const u32 w0 = (u32)warp * 32u * ITEMS + (u32)lane;  // item i of this lane: tile position w0 + 32 i
+        K key[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const u32 x = w0 + 32u * i;
+            key[i] = FULL || x < n ? kin[a + x] : K(0);
+        }
+        clear_counts();
+        __syncwarp();
+        u32 rk[ITEMS / 2];  // rank among the warp's items of the digit, two per word
+#pragma unroll
+        for (int i0 = 0; i0 < ITEMS; i0 += 2) {
+            u32 m[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int i = i0 + e;
+                const u32 d = digit_of(key[i], keymask, shift);
+                const bool valid = FULL || w0 + 32u * i < n;
+                if constexpr (STABLE) m[e] = match_digit8(d, FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, valid));
+                else m[e] = valid ? atomicAdd(wh + d, 1u) : 0u;
+            }
+            if constexpr (STABLE) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int i = i0 + e;
+                    const u32 d = digit_of(key[i], keymask, shift);
+                    const bool valid = FULL || w0 + 32u * i < n;
+                    // every lane reads the digit's count before its first lane advances it
+                    const u32 below = (u32)__popc(m[e] & lt), cnt = wh[d];
+                    __syncwarp();
+                    if (valid && below == 0u) wh[d] = cnt + (u32)__popc(m[e]);
+                    __syncwarp();
+                    m[e] = cnt + below;
+                }
+            }
+            rk[i0 / 2] = m[0] | (m[1] << 16);
+        }
+        V val[ITEMS];  // (in flight over the scan of the counts)
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const u32 x = w0 + 32u * i;
+            if constexpr (IOTA) val[i] = (V)(a + x);
+            else val[i] = FULL || x < n ? vin[a + x] : V(0);
+        }
+        __syncthreads();  // the warps' counts are known; the previous tile is written out
+        {
+            const int d = tid;
+            u32 c[WARPS], tot = 0;
+#pragma unroll
+            for (int w = 0; w < WARPS; ++w) {
+                c[w] = s_wh[w * RADIX + d];
+                tot += c[w];
+            }
+            u32 inc = tot;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 x = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += x;
+            }
+            if (lane == 31) s_scan[warp] = inc;
+            __syncthreads();
+            u32 ex = inc - tot;
+#pragma unroll
+            for (int w = 0; w < WARPS - 1; ++w) ex += w < warp ? s_scan[w] : 0u;
+            const u32 run = s_run[d];
+            s_gdst[d] = run - ex;
+            s_run[d] = run + tot;
+#pragma unroll
+            for (int w = 0; w < WARPS; ++w) {
+                s_wh[w * RADIX + d] = ex;
+                ex += c[w];
+            }
+        }
+        __syncthreads();  // first positions per (warp, digit)
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            if (FULL || w0 + 32u * i < n) {
+                const u32 pos = wh[digit_of(key[i], keymask, shift)] + ((rk[i / 2] >> (16 * (i & 1))) & 0xffffu);
+                if (DOMAGG_GUARD(pos < n, SITE_SORT_LOCAL)) {
+                    s_k[pos] = key[i];
+                    s_v[pos] = val[i];
+                }
+            }
+        }
+        __syncthreads();  // the tile in digit order
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const u32 x = (u32)tid + (u32)i * THREADS;
+            if (FULL || x < n) {
+                const K k = s_k[x];
+                const V v = s_v[x];
+                const u32 dst = s_gdst[digit_of(k, keymask, shift)] + x;
+                if (domagg_check(dst - seg_begin < seg_len, SITE_SORT_SCATTER)) {  // only fails after a timed-out wait
+                    kout[dst] = k;
+                    vout[dst] = v;
+                }
+            }
+        }
+    };
+
     for (;;) {
-        if (tid == 0) s_info[0] = atomicAdd(&ctl->tile_ctr[launch_idx], 1u);
-        for (int x = tid; x < WARPS * (RADIX + 1); x += THREADS) s_whist[x] = 0;
+        __syncthreads();  // the previous range is written out
+        if (tid == 0) s_range = atomicAdd(&ctl->tile_ctr[launch_idx], 1u);
         __syncthreads();
-        const u32 r = s_info[0];
+        const u32 r = s_range;
         if (r >= nranges) break;
         const TileLoc L = locate_range(r, seg_off, range_off, nseg, range_items);
-        // a segment whose keys have fewer digits is already in place (the
-        // barrier keeps thread 0's next claim from overwriting s_info[0]
-        // before every thread has read it)
-        if (seg_bits && (u32)pass * RADIX_BITS >= __ldg(seg_bits + L.seg)) {
-            __syncthreads();
-            continue;
-        }
-        const u32 ntile = (L.end - L.start + TILE - 1) / TILE;
-        if (tid == 0) {  // the first tile's load overlaps the range histogram
-            fence_proxy_async_smem();
-            issue(b, L.start, min(L.start + (u32)TILE, L.end));
-            pending[b] = true;
-        }
-        // 1. digit counts of the range (per-warp histograms, then summed)
+        // a segment whose keys have fewer digits is already in place
+        if (seg_bits && (u32)pass * RADIX_BITS >= __ldg(seg_bits + L.seg)) continue;
         if (range_base) {
-            for (int d = tid; d < RADIX; d += THREADS) s_run[d] = __ldg(range_base + (u64)r * RADIX + d);
+            s_run[tid] = __ldg(range_base + (u64)r * RADIX + tid);
         } else {
-            u32* wh = s_whist + warp * (RADIX + 1);
-            // evenly spread digits (see k_radix_hist): plain shared atomics
-            const bool plain = uniform && seg_bits && (int)__ldg(seg_bits + L.seg) - shift >= 5;
+            // 1. digit counts of the range
+            clear_counts();
+            __syncwarp();
             for (u32 base = L.start; base < L.end; base += (u32)THREADS * 8u) {
                 K kk[8];
 #pragma unroll
@@ -313,193 +417,34 @@ __global__ __launch_bounds__(ONESWEEP_THREADS, ONESWEEP_MIN_CTAS) void k_oneswee
                     kk[j] = x < L.end ? kin[x] : K(0);
                 }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const u32 d = digit_of(kk[j], keymask, shift);
-                    const bool valid = base + (u32)j * THREADS + (u32)tid < L.end;
-                    if (plain) {
-                        if (valid) atomicAdd(&wh[d], 1u);
-                    } else {
-                        warp_hist_add(wh, d, valid, (u32)lane);
-                    }
-                }
+                for (int j = 0; j < 8; ++j)
+                    if (base + (u32)j * THREADS + (u32)tid < L.end) atomicAdd(wh + digit_of(kk[j], keymask, shift), 1u);
             }
             __syncthreads();
-            for (int d = tid; d < RADIX; d += THREADS) {
-                u32 c = 0;
-                for (int w = 0; w < WARPS; ++w) c += s_whist[w * (RADIX + 1) + d];
-                s_dstart[d] = c;
-            }
-            __syncthreads();
-        // 2. publish the range's counts and look back over the earlier ranges
-        {
+            u32 cnt = 0;
+#pragma unroll
+            for (int w = 0; w < WARPS; ++w) cnt += s_wh[w * RADIX + tid];
+            __syncthreads();  // read before the first tile's counts
+            // 2. publish the range's counts and look back over the earlier ranges
             const u32 first_range = r - (L.start - L.seg_begin) / range_items;
-            for (int d = tid; d < RADIX; d += THREADS) {
-                const u32 cnt = s_dstart[d];
-                u64* st = status + (u64)r * RADIX + d;
-                u32 excl = 0;
-                if (L.first) {
-                    st_store(st, st_pack(epoch, ST_PREFIX, cnt));
-                } else {
-                    st_store(st, st_pack(epoch, ST_AGG, cnt));
-                    excl = lookback_u32(status, RADIX, d, r, first_range, epoch, ctl, 1u);
-                    st_store(st, st_pack(epoch, ST_PREFIX, excl + cnt));
-                }
-                s_run[d] = __ldg(digit_off + ((u64)L.seg * npass + pass) * RADIX + d) + excl;
+            u64* st = status + (u64)r * RADIX + tid;
+            u32 excl = 0;
+            if (L.first) {
+                st_store(st, st_pack(epoch, ST_PREFIX, cnt));
+            } else {
+                st_store(st, st_pack(epoch, ST_AGG, cnt));
+                excl = lookback_u32(status, RADIX, tid, r, first_range, epoch, ctl, 1u);
+                st_store(st, st_pack(epoch, ST_PREFIX, excl + cnt));
             }
-        }
+            s_run[tid] = __ldg(digit_off + ((u64)L.seg * npass + pass) * RADIX + tid) + excl;
         }
         // 3. the tiles of the range, in order
-        for (u32 j = 0; j < ntile; ++j) {
-            const u32 a = L.start + j * (u32)TILE;
-            const u32 n = min(a + (u32)TILE, L.end) - a;
-            for (int x = tid; x < WARPS * (RADIX + 1); x += THREADS) s_whist[x] = 0;
-            fence_proxy_async_smem();
-            __syncthreads();  // counters cleared; the other buffer is free
-            if (tid == 0 && j + 1 < ntile) {
-                const u32 a2 = a + (u32)TILE;
-                issue(b ^ 1, a2, min(a2 + (u32)TILE, L.end));
-                pending[b ^ 1] = true;
-            }
-            // every thread observes the completion of the copy it reads
-            if (mbar_wait_bounded(&s_bar[b], phase[b], ctl, 5u)) {
-                phase[b] ^= 1u;
-                if (tid == 0) pending[b] = false;
-            } else {
-                s_info[6] = 1u;
-            }
-            __syncthreads();
-            if (s_info[6]) break;
-            const K* bk = reinterpret_cast<const K*>(smem + b * SM::BUF) + s_info[1 + b];
-            const V* bv = reinterpret_cast<const V*>(smem + b * SM::BUF + SM::KBYTES) + s_info[3 + b];
-            // warp w ranks items [w*32*ITEMS, ...); item i of lane l at i*32 + l
-            K key[ITEMS];
-            u32 pos[ITEMS];
-            const u32 wbase = (u32)warp * 32u * ITEMS;
-            u32* wh = s_whist + warp * (RADIX + 1);
-            if (!STABLE) {
-                // any order inside a digit will do: one atomic per item
-#pragma unroll
-                for (int i = 0; i < ITEMS; ++i) {
-                    const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                    key[i] = x < n ? bk[x] : K(0);
-                    pos[i] = x < n ? atomicAdd(&wh[digit_of(key[i], keymask, shift)], 1u) : 0u;
-                }
-            } else {
-            // digit matches of all items first (independent ballots pipeline) ...
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                const bool valid = x < n;
-                key[i] = valid ? bk[x] : K(0);
-                pos[i] = match_digit8(digit_of(key[i], keymask, shift), __ballot_sync(0xffffffffu, valid));
-            }
-            // ... then, item by item, the group's leader advances the warp's
-            // count of the digit (shared-memory atomics of one warp are
-            // performed in program order) and shares the old count
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                const u32 peers = pos[i];
-                const bool valid = x < n;
-                const int leader = valid ? __ffs(peers) - 1 : lane;
-                u32 old = 0;
-                if (valid && lane == leader) old = atomicAdd(&wh[digit_of(key[i], keymask, shift)], (u32)__popc(peers));
-                pos[i] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
-            }
-            }
-            __syncthreads();
-            for (int d = tid; d < RADIX; d += THREADS) {  // exclusive over warps; tile count
-                u32 sum = 0;
-                for (int w = 0; w < WARPS; ++w) {
-                    const u32 c = s_whist[w * (RADIX + 1) + d];
-                    s_whist[w * (RADIX + 1) + d] = sum;
-                    sum += c;
-                }
-                s_dstart[d] = sum;
-            }
-            __syncthreads();
-            if (warp == 0) {  // exclusive scan of the tile counts over the digits (in place)
-                constexpr int PER = RADIX / 32;
-                u32 v[PER], sacc = 0;
-#pragma unroll
-                for (int q = 0; q < PER; ++q) {
-                    v[q] = s_dstart[lane * PER + q];
-                    sacc += v[q];
-                }
-                u32 inc = sacc;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const u32 nn = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += nn;
-                }
-                u32 ex = inc - sacc;
-#pragma unroll
-                for (int q = 0; q < PER; ++q) {
-                    s_dstart[lane * PER + q] = ex;
-                    ex += v[q];
-                }
-            }
-            __syncthreads();
-            // per (warp, digit): the warp's first local position; per digit:
-            // the global position of local index 0
-            // (then s_dstart is reused for the latter and the running
-            // positions advance by the tile's counts)
-            static_assert(THREADS == RADIX, "one thread per digit");
-            {
-                const int d = tid;
-                const u32 ds = s_dstart[d];
-                const u32 dn = d + 1 < RADIX ? s_dstart[d + 1] : n;
-                for (int w = 0; w < WARPS; ++w) s_whist[w * (RADIX + 1) + d] += ds;
-                const u32 gdst = s_run[d] - ds;
-                s_run[d] += dn - ds;
-                __syncthreads();
-                s_dstart[d] = gdst;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                if (x < n) pos[i] += wh[digit_of(key[i], keymask, shift)];
-            }
-            K* sk = reinterpret_cast<K*>(smem + b * SM::BUF);
-            V* sv = reinterpret_cast<V*>(smem + b * SM::BUF + SM::KBYTES);
-            __syncthreads();  // all keys are in registers: stage over the key buffer
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                if (x < n && DOMAGG_GUARD(pos[i] < n, SITE_SORT_LOCAL)) sk[pos[i]] = key[i];
-            }
-            V val[ITEMS];
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                val[i] = IOTA ? (V)(a + x) : (x < n ? bv[x] : V(0));
-            }
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const u32 x = wbase + (u32)i * 32u + (u32)lane;
-                if (x < n && DOMAGG_GUARD(pos[i] < n, SITE_SORT_LOCAL)) sv[pos[i]] = val[i];
-            }
-            __syncthreads();
-            const u32 seg_len = L.seg_end - L.seg_begin;
-            for (u32 x = tid; x < n; x += THREADS) {
-                const K k = sk[x];
-                const u32 dst = s_dstart[digit_of(k, keymask, shift)] + x;  // (global position of index 0)
-                if (domagg_check(dst - L.seg_begin < seg_len, SITE_SORT_SCATTER)) {  // only fails after a timed-out wait
-                    kout[dst] = k;
-                    vout[dst] = sv[x];
-                }
-            }
-            b ^= 1;
+        const u32 seg_len = L.seg_end - L.seg_begin;
+        for (u32 a = L.start; a < L.end; a += (u32)TILE) {
+            const u32 n = min((u32)TILE, L.end - a);
+            if (n == (u32)TILE) do_tile(std::true_type(), a, n, L.seg_begin, seg_len);
+            else do_tile(std::false_type(), a, n, L.seg_begin, seg_len);
         }
-        __syncthreads();
-        if (s_info[6]) break;
-    }
-    // a copy may still be in flight if a wait ran out: wait for it (bounded)
-    if (tid == 0) {
-        for (int bb = 0; bb < 2; ++bb)
-            if (pending[bb]) mbar_wait_bounded(&s_bar[bb], phase[bb], ctl, 6u);
     }
 }
 

@@ -27,18 +27,36 @@ static u64 resident_ctas(size_t smem) {
     return (u64)std::max(sms, 1) * (u64)per_sm;
 }
 
+// From this many ranges on, a pass takes its ranges' positions from two small
+// launches (count, scan) instead of a look-back: all resident CTAs publish
+// their counts at once, so the walks over the first wave's aggregates were
+// half of the pass's instructions (225 per item against 110 without, at
+// 6.3e6 pairs; the whole m = 3 forward at 2^21 per side 13.1 -> 12.9 ms, the
+// mixed batch 23.5 -> 23.1).  Below, the launches' own latency is the larger
+// part (m = 2, 1.7e5 points: 390 us with the look-back, 412 without).
+#ifndef DOMAGG_RANGE_SCAN_MIN
+#define DOMAGG_RANGE_SCAN_MIN 300
+#endif
+constexpr u64 RANGE_SCAN_MIN = DOMAGG_RANGE_SCAN_MIN;
+static void range_bases(Launcher& L, const SortSpace& sp, u64 nranges, int npass, int pass, u32* range_cnt) {
+    const u32* off = sp.digit_off + (size_t)pass * RADIX;
+    const dim3 grid(sp.nseg, RADIX / 32);
+    if (nranges >= 64ull * sp.nseg) k_range_bases<32><<<grid, 32 * 32, 0, L.stream>>>(sp.tile_off, off, npass, range_cnt);
+    else k_range_bases<1><<<grid, 32, 0, L.stream>>>(sp.tile_off, off, npass, range_cnt);
+}
+
 template <typename K, typename V, bool IOTA, bool STABLE>
 static void launch_pass(Launcher& L, unsigned grid, size_t smem, K* kin, V* vin, K* kout, V* vout,
                         const SortSpace& sp, u32 range_items, const u32* seg_bits, const u32* range_base, int npass,
-                        int p, K keymask, int li, bool uniform) {
+                        int p, K keymask, int li) {
     k_onesweep<K, V, IOTA, STABLE><<<grid, ONESWEEP_THREADS, smem, L.stream>>>(
         kin, vin, kout, vout, sp.seg_off, sp.tile_off, sp.nseg, range_items, seg_bits, range_base, sp.digit_off,
-        npass, p, p * RADIX_BITS, keymask, sp.status, L.ctl, li, uniform ? 1 : 0);
+        npass, p, p * RADIX_BITS, keymask, sp.status, L.ctl, li);
 }
 
 template <typename K, typename V>
 int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool iota, int total_bits, K keymask,
-               int kind_hist, int kind_pass, const u32* seg_bits, bool stable, bool uniform) {
+               int kind_hist, int kind_pass, const u32* seg_bits, bool stable) {
     constexpr u32 TILE = ONESWEEP_THREADS * onesweep_items<K, V>();
     static_assert(TILE >= SORT_MIN_TILE, "status words are sized for SORT_MIN_TILE");
     const int npass = (total_bits + RADIX_BITS - 1) / RADIX_BITS;
@@ -91,16 +109,14 @@ int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool io
     cudaMemsetAsync(sp.hist, 0, hist_bytes, L.stream);
     L.start(kind_hist, sp.n_items * sizeof(K));
     k_radix_hist<K><<<(unsigned)nranges, 256, hist_smem, L.stream>>>(
-        keys[0], sp.seg_off, sp.tile_off, sp.nseg, range_items, npass, 0, keymask, sp.hist, range_base, seg_bits,
-        uniform ? 1 : 0);
+        keys[0], sp.seg_off, sp.tile_off, sp.nseg, range_items, npass, 0, keymask, sp.hist, range_base, seg_bits);
     L.stop();
     L.start(KIND_SMALL, 0.0);
     k_radix_offsets<<<sp.nseg * npass, RADIX, 0, L.stream>>>(sp.hist, sp.seg_off, npass, sp.digit_off);
     L.stop();
     if (range_base) {
         L.start(KIND_SMALL, 0.0);
-        k_range_bases<<<dim3(sp.nseg, RADIX / 32), RB_WARPS * 32, 0, L.stream>>>(sp.tile_off, sp.digit_off, npass,
-                                                                                  range_base);
+        range_bases(L, sp, nranges, npass, 0, range_base);
         L.stop();
     }
     int cur = 0;
@@ -123,17 +139,30 @@ int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool io
             for (size_t sgi = 0; sgi < sp.seg_sizes->size(); ++sgi)
                 if ((u32)p * RADIX_BITS < (*sp.seg_bits_host)[sgi]) moved += (double)(*sp.seg_sizes)[sgi];
         }
+        // later passes: the ranges' counts and bases as launches of their own
+        // where there are many ranges (see RANGE_SCAN_MIN)
+        const u32* rb = p == 0 ? range_base : nullptr;
+        if (p > 0 && nranges >= RANGE_SCAN_MIN && sp.range_scratch && nranges <= sp.range_scratch_ranges) {
+            L.start(kind_hist, moved * sizeof(K));
+            k_range_count<K><<<(unsigned)nranges, 256, 0, L.stream>>>(keys[cur], sp.seg_off, sp.tile_off, sp.nseg,
+                                                                     range_items, p * RADIX_BITS, keymask,
+                                                                     sp.range_scratch);
+            L.stop();
+            L.start(KIND_SMALL, 0.0);
+            range_bases(L, sp, nranges, npass, p, sp.range_scratch);
+            L.stop();
+            rb = sp.range_scratch;
+        }
         const double vbytes = (iota && p == 0) ? sizeof(V) : 2.0 * sizeof(V);
         L.start(kind_pass, moved * (2.0 * sizeof(K) + vbytes));
-        const u32* rb = p == 0 ? range_base : nullptr;
         K *ki = keys[cur], *ko = keys[cur ^ 1];
         V *vi = vals[cur], *vo = vals[cur ^ 1];
         if (iota && p == 0) {
-            if (stable) launch_pass<K, V, true, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li, uniform);
-            else launch_pass<K, V, true, false>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li, uniform);
+            if (stable) launch_pass<K, V, true, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
+            else launch_pass<K, V, true, false>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
         } else {
-            if (stable) launch_pass<K, V, false, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li, uniform);
-            else launch_pass<K, V, false, false>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li, uniform);
+            if (stable) launch_pass<K, V, false, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
+            else launch_pass<K, V, false, false>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
         }
         L.stop();
         cur ^= 1;
@@ -159,10 +188,10 @@ u32 bounds_site_sort(bool clear) {
 }
 
 template int sort_pairs<u32, u32>(Launcher&, const SortSpace&, u32**, u32**, bool, int, u32, int, int,
-                                     const u32*, bool, bool);
+                                     const u32*, bool);
 template int sort_pairs<u64, u32>(Launcher&, const SortSpace&, u64**, u32**, bool, int, u64, int, int,
-                                     const u32*, bool, bool);
+                                     const u32*, bool);
 template int sort_pairs<u32, u64>(Launcher&, const SortSpace&, u32**, u64**, bool, int, u32, int, int,
-                                     const u32*, bool, bool);
+                                     const u32*, bool);
 
 }  // namespace domagg
