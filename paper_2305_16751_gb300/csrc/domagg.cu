@@ -708,7 +708,9 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     // m = 2 the levels above the groups of ranks that k_group takes)
     L.start(KIND_SMALL, 0.0);
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,
-                                            govf, M == 3 ? G3_CAP : GROUP_CAP, use_groups ? h->group_bits : 0,
+                                            govf, M == 3 ? G3_CAP : GROUP_CAP,
+                                            M == 3 ? g3_avg(N, h->no_alloc || h->max_ws > 0) : 0xffffffffu,
+                                            use_groups ? h->group_bits : 0,
                                             use_top ? h->top_bits : 0);
     cudaMemsetAsync(rec_all, 0, sizeof(unsigned long long) * k, stream);
     L.stop();
@@ -897,14 +899,14 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         if (!planned) {
             gb_host.resize(k);
             for (int s = 0; s < k; ++s) {
-                gb_host[s] = inst[s].gS ? inst[s].b[0] - inst[s].gS : 0u;
+                gb_host[s] = inst[s].gS ? inst[s].b[0] - inst[s].gS + (M == 3 ? 1u : 0u) : 0u;  // (m = 3: and the role)
                 gbits_max = std::max(gbits_max, (int)gb_host[s]);
             }
         } else {  // bound: ranks below 2n (a non-strict first coordinate doubles them)
             for (int s = 0; s < k; ++s) {
                 int bb = 0;
                 while (bb < 32 && (1ull << bb) < 2 * pt_sizes[s]) ++bb;
-                gbits_max = std::max(gbits_max, bb);
+                gbits_max = std::max(gbits_max, bb + (M == 3 ? 1 : 0));
             }
         }
         SortSpace gs{d_pt_offs, k, planned ? nullptr : &pt_sizes, d_sort_tiles, hist, digit_off,
@@ -927,13 +929,11 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         } else {
             // m = 3: the group-sorted rank and position, the second rank and
             // (data) the weight gathered by position, a partial per query
-            constexpr size_t gsm = G3Smem<Acc>::TOTAL;
-            if (!L.frozen) cudaFuncSetAttribute(k_group3<Op, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
             L.start(KIND_GROUP, (double)N * (8.0 + 4.0) + (double)(N - NQ) * (WT == 3 ? 0.0 : sizeof(W)) +
                                     (double)NQ * sizeof(Part));
-            k_group3<Op, WT><<<(unsigned)h->sms, G3_THREADS, gsm, stream>>>(d_inst, k, gslot, rstart, gval[0],
-                                                                            gval[1], pr1, (const W*)P[18], gacc,
-                                                                            h->ctl, li);
+            k_group3<Op, WT><<<2u * (unsigned)h->sms, PAIR_THREADS, 0, stream>>>(d_inst, k, gslot, rstart, gval[0],
+                                                                                 gval[1], pr1, (const W*)P[18], gacc,
+                                                                                 h->ctl, li);
             L.stop();
         }
     }

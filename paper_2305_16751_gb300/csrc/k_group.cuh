@@ -49,8 +49,8 @@ __host__ __device__ constexpr size_t group_smem_bytes() {
 
 // Per instance (one block each): the largest gS <= min(GROUP_MAX_BITS, b0)
 // whose groups of 2^gS ranks that hold more than `cap` points each (too
-// many for shared memory: heavy ties) hold at most a quarter of the points,
-// and the number of groups G (m = 2: k_group; m = 3: k_group3); gS = 0 (no
+// many for shared memory: heavy ties) hold at most a quarter of the points
+// and which hold at most `avg` points on average, and the number of groups G (m = 2: k_group; m = 3: k_group3); gS = 0 (no
 // level in groups) if no width qualifies, or if the instance takes another
 // path.  govf[pt_off + g] = 1 marks this shard's groups that overflow: their
 // points' levels below gS go through the records in HBM.  With top_bits > 0, the
@@ -61,11 +61,12 @@ __host__ __device__ constexpr size_t group_smem_bytes() {
 // first point of every (undoubled) rank, and n at index U.  A non-strict
 // first coordinate doubles the ranks (2r for data, 2r+1 for queries), so a
 // group of 2^gS ranks is 2^(gS-1) undoubled ranks.  Also writes gbits[s],
-// the bits of the group id (b0 - gS) the group sort sorts.
+// the bits the group sort sorts: the group id's (b0 - gS) and, for m = 3, the
+// role's.
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
-                                                    u32 cap, int max_bits, int top_bits) {
+                                                    u32 cap, u32 avg, int max_bits, int top_bits) {
     __shared__ u32 s_ovf[32];
     __shared__ u32 s_done;
     const int s = blockIdx.x;
@@ -93,7 +94,7 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
         if (threadIdx.x == 0) {
             u32 t = 0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_ovf[w];
-            s_done = t <= n / 4u ? 1u : 0u;
+            s_done = (t <= n / 4u && n <= (u64)avg * g_n) ? 1u : 0u;
         }
         __syncthreads();
         const bool ok = s_done != 0u;
@@ -114,7 +115,7 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
     if (threadIdx.x == 0) {
         I.gS = chosen;
         I.G = chosen ? G : 0u;
-        if (gbits) gbits[s] = chosen ? b0 - chosen : 0u;
+        if (gbits) gbits[s] = chosen ? b0 - chosen + (M == 3 ? 1u : 0u) : 0u;
         // the levels >= gS of this shard: from tS up per tile (k_top), below
         // tS through the records in HBM
         const u32 nlev = M == 1 ? 1u : b0;

@@ -475,7 +475,7 @@ __global__ __launch_bounds__(256) void k_count_scan(
             // for m = 3, its position x)
             if ((M == 2 || M == 3) && gkey && I.gS) {
                 const u32 pv = (q || WT == 1 || M == 3) ? x : wbits;
-                gkey[x] = a >> I.gS;
+                gkey[x] = M == 3 ? ((a >> I.gS) << 1) | (q ? 1u : 0u) : a >> I.gS;  // (m = 3: data first)
                 gval[x] = ((u64)(q ? (a | QUERY_BIT) : a) << 32) | (u64)pv;
             }
         }
