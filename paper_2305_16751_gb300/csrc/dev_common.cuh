@@ -67,7 +67,8 @@ struct Inst {
     u32 gS, G;
     // m = 2: rank levels tS .. b0-1 (at most TOP_MAX_BITS) are taken per tile
     // of points in the order of the last coordinate (k_top); topmask: those
-    // of this call's shard (bit lv; device-computed)
+    // of this call's shard (bit lv; device-computed).  m = 3: topmask holds the
+    // levels taken by items (k_items.cuh), if any
     u32 tS, topmask;
     // levels of the first rank whose records this call takes through HBM
     // (bit lv; device-computed), and the call's shard of the flat map: shard

@@ -22,6 +22,7 @@
 #include "k_radix.cuh"
 #include "k_group.cuh"
 #include "k_group3.cuh"
+#include "k_items.cuh"
 #include "k_records.cuh"
 #include "k_top.cuh"
 #include "k_wavelet.cuh"
@@ -75,6 +76,15 @@ struct domagg_ctx {
     Ctl ctl_host{};            // the control block as last read back
     u64 pair_T_seen[4] = {0, 0, 0, 0};  // Ctl::pair_T already accounted for
     bool use_pairs = true;     // tuning knob "pairs"
+    // m = 3: the levels above the groups as m = 2 problems (k_items.cuh), on a
+    // handle of their own; tuning knob "nodes" (1: by size, 2: always)
+    DevBuf items;
+    domagg_ctx* sub = nullptr;
+    int nodes = 1;
+    // on that handle: the point phase's input, ready-made (ranked keys of at
+    // most pre_bits bits, by point; the order of the last coordinate)
+    u32 *pre_keys = nullptr, *pre_perm = nullptr;
+    int pre_bits = 32;
     void* h_pin = nullptr;
     size_t h_pin_cap = 0;
     std::string err;
@@ -112,7 +122,8 @@ struct domagg_ctx {
     int rank_windows = 0;
 
     size_t held() const {
-        return pts.cap + recs.cap + st_multi.cap + st_seg.cap + stage.cap + st_wv.cap + pairs.cap + st_pairs.cap;
+        return pts.cap + recs.cap + st_multi.cap + st_seg.cap + stage.cap + st_wv.cap + pairs.cap + st_pairs.cap +
+               items.cap + (sub ? sub->held() : 0);
     }
 };
 
@@ -224,30 +235,37 @@ struct OpTraits;
 template <>
 struct OpTraits<OpSumF32> {
     static constexpr int WT = 2;
+    static constexpr domagg_op OP = DOMAGG_SUM;
 };
 template <>
 struct OpTraits<OpSumI64> {
     static constexpr int WT = 1;
+    static constexpr domagg_op OP = DOMAGG_SUM;
 };
 template <>
 struct OpTraits<OpMaxI32> {
     static constexpr int WT = 0;
+    static constexpr domagg_op OP = DOMAGG_MAX;
 };
 template <>
 struct OpTraits<OpMaxF32> {
     static constexpr int WT = 2;
+    static constexpr domagg_op OP = DOMAGG_MAX;
 };
 template <>
 struct OpTraits<OpMinI32> {
     static constexpr int WT = 0;
+    static constexpr domagg_op OP = DOMAGG_MIN;
 };
 template <>
 struct OpTraits<OpMinF32> {
     static constexpr int WT = 2;
+    static constexpr domagg_op OP = DOMAGG_MIN;
 };
 template <>
 struct OpTraits<OpCount> {
     static constexpr int WT = 3;
+    static constexpr domagg_op OP = DOMAGG_COUNT;
 };
 
 // Resets the look-back epoch and the status words when the epoch counter
@@ -388,9 +406,216 @@ domagg_status run_wavelet(domagg_ctx* h, std::vector<Inst>& inst, Inst* d_inst, 
     return DOMAGG_OK;
 }
 
+domagg_status dispatch(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype ct, domagg_dtype wt,
+                       domagg_op op, bool negate, cudaStream_t s, const std::vector<PlannedChunk>* pl = nullptr,
+                       bool pairs = true, bool items = true);
+
+// Pinned memory for tables (contents are not kept).
+domagg_status grow_pinned_tables(domagg_ctx* h, size_t bytes) {
+    if (h->h_pair_cap >= bytes) return DOMAGG_OK;
+    if (h->h_pair) {
+        cudaDeviceSynchronize();
+        cudaFreeHost(h->h_pair);
+    }
+    h->h_pair = nullptr;
+    h->h_pair_cap = 0;
+    const size_t want = std::max<size_t>(bytes + bytes / 2, 1 << 16);
+    if (cudaMallocHost(&h->h_pair, want) != cudaSuccess) {
+        cudaGetLastError();
+        h->h_pair = nullptr;
+        return fail(h, DOMAGG_ERR_OOM, "pinned memory for tables");
+    }
+    h->h_pair_cap = want;
+    return DOMAGG_OK;
+}
+
+// m = 3: what the items' stage reads of the point phase, and what it leaves:
+// a partial per (level, query item), at qseg[instance][level] + the query's
+// place in the level.
+constexpr u64 ITEM_MAX_NODES = 1u << 17, ITEM_MIN_POINTS = 1u << 20;
+struct ItemStage {
+    int k;
+    const std::vector<u32>*lvl, *qlvl;  // items and query items per (instance, level)
+    u64 nchunk;
+    const u32 *chunk_off, *pt_offs, *pt_tiles, *pr0, *pr1, *chunk_base, *qchunk_base, *tile_excl;
+    const Inst* d_inst;
+    const void* pw;
+    void* part = nullptr;
+    u32 n_part = 0;
+    const u32* qseg = nullptr;
+};
+// DOMAGG_ERR_OOM: too many nodes or no room; the caller takes the records.
+template <class Op>
+domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& inst, ItemStage& S) {
+    typedef typename Op::W W;
+    typedef typename Op::Out Out;
+    typedef typename Op::Part Part;
+    constexpr int WT = OpTraits<Op>::WT;
+    constexpr size_t WB = WT == 3 ? 0 : sizeof(W);
+    const cudaStream_t stream = L.stream;
+    const int k = S.k;
+    // segments: the levels of every instance, with items
+    std::vector<u32> so, sbits, sbase((size_t)k * LMAX, 0), qsbase((size_t)k * LMAX, 0);
+    std::vector<u64> sizes;
+    u64 T = 0, Q = 0, nodes = 0;
+    int bits_max = 0, r1_bits = 0;
+    for (int s = 0; s < k; ++s) r1_bits = std::max(r1_bits, (int)inst[s].b[1]);
+    for (int s = 0; s < k; ++s)
+        for (u32 lv = 0; lv < LMAX; ++lv) {
+            const u64 n = (*S.lvl)[(size_t)s * LMAX + lv];
+            sbase[(size_t)s * LMAX + lv] = (u32)T;
+            qsbase[(size_t)s * LMAX + lv] = (u32)Q;
+            if (n == 0) continue;
+            const u32 b = inst[s].b[0] - 1u - lv;  // bits of the level's node
+            so.push_back((u32)T);
+            sbits.push_back(b);
+            sizes.push_back(n);
+            bits_max = std::max(bits_max, (int)b);
+            nodes += std::min<u64>(n, 1ull << b);
+            T += n;
+            Q += (*S.qlvl)[(size_t)s * LMAX + lv];
+        }
+    so.push_back((u32)T);
+    if (T == 0) return DOMAGG_OK;
+    if (T >= (1ull << 31) || nodes > ITEM_MAX_NODES) return fail(h, DOMAGG_ERR_OOM, "too many nodes");
+    const size_t nseg = sizes.size();
+    const int npass = (bits_max + RADIX_BITS - 1) / RADIX_BITS;
+    const u64 ntile = tiles_of(sizes, ITEM_TILE), nrb = sort_range_bound(sizes);
+    const size_t hist_words = nseg * std::max(npass, 1) * RADIX;
+    const size_t up_words = (nseg + 1) + nseg + 2 * (size_t)k * LMAX + 2;
+    void* R[22];
+    auto carve = [&](Carver& c) {
+        R[0] = c.take<u32>(up_words);
+        R[1] = c.take<u32>(nseg + 1);  // the sort's ranges
+        R[2] = c.take<u32>(nseg + 1);  // the node search's tiles
+        R[3] = c.take<u32>(T);
+        R[4] = c.take<u32>(T);
+        R[5] = c.take<u64>(T);
+        R[6] = c.take<u64>(T);
+        R[7] = c.take<u32>(hist_words);
+        R[8] = c.take<u32>(hist_words);
+        R[9] = c.take<u32>((size_t)nrb * RADIX);
+        R[10] = c.take<u32>(ntile + 1);
+        R[11] = c.take<u32>(ntile + 1);
+        R[12] = c.take<u32>(nodes + 1);
+        R[13] = c.take<u32>(nodes + 1);
+        R[14] = c.take<u32>(T);  // the nodes' problems: ranked keys, permutation
+        R[15] = c.take<u32>(Q);
+        R[16] = c.take<u32>(T);
+        R[17] = c.take<char>((size_t)(T - Q) * WB);
+        R[18] = c.take<Out>(Q);
+        R[19] = c.take<Part>(Q);
+    };
+    Carver c0(nullptr);
+    carve(c0);
+    domagg_status st = grow(h, h->items, c0.off);
+    if (!st) st = grow(h, h->st_multi, (size_t)tiles_of(sizes, SORT_MIN_TILE) * RADIX * sizeof(u64), true);
+    if (!st) st = grow_pinned_tables(h, sizeof(u32) * (up_words + 2 * nodes + 1));
+    if (!st && !h->sub) {
+        st = domagg_create(&h->sub, h->device, 0);
+        if (st) return fail(h, DOMAGG_ERR_OOM, "the nodes' handle");
+    }
+    if (st) return st;
+    Carver c1(h->items.p);
+    carve(c1);
+    u32* hp = (u32*)h->h_pair;
+    u32* w = hp;
+    auto put = [&](const std::vector<u32>& v) {
+        memcpy(w, v.data(), sizeof(u32) * v.size());
+        w += v.size();
+    };
+    put(so);
+    put(sbits);
+    put(sbase);
+    put(qsbase);
+    w[0] = 0;
+    w[1] = (u32)ntile + 1u;
+    u32 *d_so = (u32*)R[0], *d_sbits = d_so + nseg + 1, *d_sbase = d_sbits + nseg, *d_qsbase = d_sbase + (size_t)k * LMAX,
+        *d_one = d_qsbase + (size_t)k * LMAX;
+    u32 *keys[2] = {(u32*)R[3], (u32*)R[4]}, *cnt_h = (u32*)R[10], *cnt_q = (u32*)R[11];
+    u64* pays[2] = {(u64*)R[5], (u64*)R[6]};
+    cudaMemcpyAsync(d_so, hp, sizeof(u32) * up_words, cudaMemcpyHostToDevice, stream);
+    cudaMemsetAsync(cnt_h, 0, sizeof(u32) * (ntile + 1), stream);
+    cudaMemsetAsync(cnt_q, 0, sizeof(u32) * (ntile + 1), stream);
+    const unsigned grid = (unsigned)std::min<u64>((S.nchunk + 7) / 8, (u64)h->sms * L.blocks_per_sm);
+    L.start(KIND_EXPAND, (double)S.nchunk * 32 * 8 + (double)T * 12);
+    k_item_expand<<<grid, 256, 0, stream>>>(S.chunk_off, k, S.pt_offs, S.pr0, S.pr1, S.chunk_base, S.qchunk_base,
+                                            S.pt_tiles, S.tile_excl, S.d_inst, d_sbase, d_qsbase, (u32)T, keys[0],
+                                            pays[0]);
+    L.stop();
+    SortSpace rs{d_so, (int)nseg, &sizes, (u32*)R[1], (u32*)R[7], (u32*)R[8], (u64*)h->st_multi.p, (double)T,
+                 (u32*)R[9], nrb, &sbits, T};
+    if (npass > 0)
+        sort_pairs<u32, u64>(L, rs, keys, pays, false, bits_max, ~QUERY_BIT, KIND_HIST_RECORDS, KIND_SORT_RECORDS,
+                             d_sbits, true);
+    L.start(KIND_SMALL, 0.0);
+    k_make_tiles<<<1, 1024, 0, stream>>>(d_so, (int)nseg, ITEM_TILE, (u32*)R[2]);
+    L.stop();
+    L.start(KIND_SMALL, (double)T * 4);
+    k_item_heads<<<(unsigned)ntile, 256, 0, stream>>>(keys[0], keys[1], d_so, (u32*)R[2], (int)nseg, d_sbits, cnt_h,
+                                                      cnt_q);
+    L.stop();
+    L.start(KIND_SMALL, 0.0);
+    k_tile_exscan<<<1, 1024, 0, stream>>>(d_one, 1, cnt_h);  // one segment of ntile + 1 counts
+    k_tile_exscan<<<1, 1024, 0, stream>>>(d_one, 1, cnt_q);
+    L.stop();
+    L.start(KIND_SMALL, (double)T * 4);
+    k_item_starts<<<(unsigned)ntile, 256, 0, stream>>>(keys[0], keys[1], d_so, (u32*)R[2], (int)nseg, d_sbits, cnt_h,
+                                                       cnt_q, (u32)nodes, (u32)T, (u32)Q, (u32*)R[12], (u32*)R[13]);
+    L.stop();
+    L.start(KIND_EXPAND, (double)T * (12 + 8 + WB));
+    k_item_place<Op, WT><<<(unsigned)ntile, 256, 0, stream>>>(
+        keys[0], keys[1], pays[0], pays[1], d_so, (u32*)R[2], (int)nseg, d_sbits, cnt_h, cnt_q, (const W*)S.pw,
+        (u32)nodes, (u32)T, (const u32*)R[12], (const u32*)R[13], (u32*)R[14], (u32*)R[16], (u32*)R[15], (W*)R[17]);
+    L.stop();
+    // the nodes' sizes
+    u32 *h_cnt = hp + up_words, *h_start = h_cnt + 1, *h_q = h_start + nodes;
+    L.start(KIND_D2H, 0.0);
+    cudaMemcpyAsync(h_cnt, cnt_h + ntile, sizeof(u32), cudaMemcpyDeviceToHost, stream);
+    cudaMemcpyAsync(h_start, R[12], sizeof(u32) * nodes, cudaMemcpyDeviceToHost, stream);
+    cudaMemcpyAsync(h_q, R[13], sizeof(u32) * nodes, cudaMemcpyDeviceToHost, stream);
+    L.stop();
+    cudaError_t e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "items");
+    const u64 nn = std::min<u64>(h_cnt[0], nodes);
+    std::vector<Inst> sub;
+    sub.reserve(nn);
+    for (u64 i = 0; i < nn; ++i) {
+        const u64 a = h_start[i], qa = h_q[i], b = i + 1 < nn ? h_start[i + 1] : T, qb = i + 1 < nn ? h_q[i + 1] : Q;
+        const u64 nQ = qb - qa, nD = (b - a) - nQ, da = a - qa;
+        Inst I;  // (its points are [a, b) of the keys and the permutation: none is left out)
+        memset(&I, 0, sizeof(I));
+        I.dw = WT == 3 ? nullptr : (const char*)R[17] + da * WB;
+        I.out = (Out*)R[18] + qa;
+        I.nD = (u32)nD;
+        I.nQ = (u32)nQ;
+        sub.push_back(I);
+    }
+    const unsigned qgrid = (unsigned)((Q + 255) / 256);
+    if (!sub.empty()) {
+        h->sub->timing = h->timing;
+        const domagg_dtype wt = WT == 0 ? DOMAGG_I32 : (WT == 2 ? DOMAGG_F32 : DOMAGG_I64);
+        h->sub->pre_keys = (u32*)R[14];
+        h->sub->pre_perm = (u32*)R[16];
+        h->sub->pre_bits = std::max(1, r1_bits);
+        st = dispatch(h->sub, 2, sub, DOMAGG_I32, wt, OpTraits<Op>::OP, false, stream, nullptr, false);
+        h->sub->pre_keys = h->sub->pre_perm = nullptr;
+        if (st) return fail(h, st, "nodes: " + h->sub->err);
+    }
+    if (Q > 0) {
+        L.start(KIND_REDUCE, (double)Q * (sizeof(Out) + 4 + sizeof(Part)));
+        k_item_out<Op><<<qgrid, 256, 0, stream>>>((const Out*)R[18], (const u32*)R[15], (u32)Q, (Part*)R[19]);
+        L.stop();
+    }
+    S.part = R[19];
+    S.n_part = (u32)Q;
+    S.qseg = d_qsbase;
+    return DOMAGG_OK;
+}
+
 template <int M, class Op, bool F32>
 domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStream_t stream,
-                  const std::vector<PlannedChunk>* planned = nullptr) {
+                  const std::vector<PlannedChunk>* planned = nullptr, bool items = false) {
     typedef typename std::conditional<M >= 3, u64, u32>::type K;
     typedef typename Op::Pay Pay;  // 32 bits: the weight's bits, a weight position (GATHER) or a slot
     typedef typename Op::W W;      // a weight in the order of the last coordinate
@@ -487,7 +712,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         // scratch of the sorts that run beside the first (chain 1: the last
         // coordinate; chain 2: the second rank coordinate), when overlapping
         for (int ch = 1; ch <= 2; ++ch) {
-            const bool used = h->overlap && (ch == 1 || M >= 3);
+            const bool used = h->overlap && !h->pre_keys && (ch == 1 || M >= 3);
             const u64 n = used ? N : 0, kk = used ? (u64)k : 0;
             P[29 + (ch - 1) * 8 + 0] = c.take<u32>(n);                                  // key ping-pong
             P[29 + (ch - 1) * 8 + 1] = c.take<u32>(n);                                  // values A
@@ -523,8 +748,14 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         // record of the flat map (a statistic)
         P[57] = c.take<unsigned char>(grp ? N : 0);
         P[58] = c.take<unsigned long long>(k);
+        // m = 3, the levels above the groups by items: their counts
+        P[59] = c.take<u32>(items ? (size_t)NC * LMAX : 0);
+        P[60] = c.take<u32>(items ? (size_t)NC * LMAX : 0);
+        P[61] = c.take<u32>(items ? (size_t)ntp * CS_COUNTERS : 0);
+        P[62] = c.take<u32>(items ? (size_t)k * LMAX : 0);
+        P[63] = c.take<u32>(items ? (size_t)k * LMAX : 0);
     };
-    void* P[59];
+    void* P[64];
     {
         Carver c(nullptr);
         carve_points(c, P);
@@ -565,9 +796,10 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     const size_t lvl_pos = (up_bytes + 63) & ~(size_t)63;                          // level totals (read back)
     const size_t rec_pos = (lvl_pos + 2 * sizeof(u32) * k * LMAX + 63) & ~(size_t)63;  // records per instance (read back)
     const size_t ctl_pos = (rec_pos + sizeof(unsigned long long) * k + 63) & ~(size_t)63;  // control block (read back)
+    const size_t item_pos = (ctl_pos + sizeof(Ctl) + 63) & ~(size_t)63;                    // item totals (read back)
     char* hp = nullptr;
     if (!planned) {
-        domagg_status st = grow_pinned(h, ctl_pos + sizeof(Ctl) + 64);
+        domagg_status st = grow_pinned(h, item_pos + (items ? 2 * sizeof(u32) * k * LMAX : 0) + 64);
         if (st) return st;
         hp = (char*)h->h_pin;
         memcpy(hp, inst.data(), sizeof(Inst) * k);
@@ -610,11 +842,15 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     k_make_tiles<<<1, 1024, 0, stream>>>(d_pt_offs, k, POINT_TILE, d_pt_tiles);
     L.stop();
 
+    // (m = 2, the nodes of m = 3: keys and permutation are given)
+    const bool pre = M == 2 && h->pre_keys != nullptr;
     // ---- keys (instruction 0 and 5i-4)
-    L.start(KIND_ENCODE, (double)N * M * 4 * 2);
-    k_encode<M, F32><<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(d_inst, d_pt_offs, k, (u32)N, rk0, rk1, rk2, lk,
-                                                                      negate ? 1 : 0, h->ctl);
-    L.stop();
+    if (!pre) L.start(KIND_ENCODE, (double)N * M * 4 * 2);
+    if (!pre) {
+        k_encode<M, F32><<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(d_inst, d_pt_offs, k, (u32)N, rk0, rk1, rk2,
+                                                                          lk, negate ? 1 : 0, h->ctl);
+        L.stop();
+    }
 
     // ---- the point-phase sorts (5i-3 .. 5i, 5m+i, and the Sec. 5 order of the
     // last coordinate).  They are independent: with overlap, the last
@@ -639,11 +875,11 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         L.stream = C.stream;
         SortSpace sp{d_pt_offs, k, &pt_sizes, C.tiles, C.hist, C.digit, C.status, (double)N, C.range,
                      sort_range_bound(pt_sizes)};
-        u32* keys[2] = {i == 0 ? rk0 : (i == 1 ? rk1 : rk2), C.kalt};
+        u32* keys[2] = {pre ? h->pre_keys : (i == 0 ? rk0 : (i == 1 ? rk1 : rk2)), C.kalt};
         u32* vals[2] = {C.vA, C.vB};
         // only the sorted key sequence matters for dense ranks: any order of equal digits
-        const int cur = sort_pairs<u32, u32>(L, sp, keys, vals, true, 32, 0xffffffffu, KIND_HIST_POINTS,
-                                             KIND_SORT_POINTS, nullptr, false);
+        const int cur = sort_pairs<u32, u32>(L, sp, keys, vals, true, pre ? h->pre_bits : 32, 0xffffffffu,
+                                             KIND_HIST_POINTS, KIND_SORT_POINTS, nullptr, false);
         L.start(KIND_RANK, (double)N * 4);
         k_rank_count<SCAN_THREADS, SCAN_ITEMS><<<(unsigned)ntp, SCAN_THREADS, 0, C.stream>>>(keys[cur], d_pt_offs,
                                                                                           d_pt_tiles, k, C.tile_cnt);
@@ -677,7 +913,10 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         return vals[cur];
     };
     u32* perm;
-    if (h->overlap) {
+    if (pre) {
+        rank_dim(0, chain(0));
+        perm = h->pre_perm;
+    } else if (h->overlap) {
         cudaEventRecord(h->ev_fork, stream);
         cudaStreamWaitEvent(h->aux[0], h->ev_fork, 0);
         if (M >= 3) cudaStreamWaitEvent(h->aux[1], h->ev_fork, 0);
@@ -711,7 +950,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                                             govf, M == 3 ? G3_CAP : GROUP_CAP,
                                             M == 3 ? g3_avg(N, h->no_alloc || h->max_ws > 0) : 0xffffffffu,
                                             use_groups ? h->group_bits : 0,
-                                            use_top ? h->top_bits : 0);
+                                            use_top ? h->top_bits : 0, items ? 1 : 0);
     cudaMemsetAsync(rec_all, 0, sizeof(unsigned long long) * k, stream);
     L.stop();
     // ---- count / offset scan of the flat map, per level
@@ -728,6 +967,16 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             d_pt_tiles, k, (u32*)P[25], lvl_tot, qlvl_tot, h->ctl);
         L.stop();
     }
+    if (items) {
+        L.start(KIND_COUNT_SCAN, (double)N * 4 + (double)NC * 8 * LMAX);
+        k_item_count<<<(unsigned)ntp, 256, 0, stream>>>(d_pt_offs, d_pt_tiles, k, d_chunk_off, pr0, d_inst,
+                                                        (u32*)P[59], (u32*)P[60], (u32*)P[61]);
+        L.stop();
+        L.start(KIND_SMALL, 0.0);
+        k_tile_exscan_counters<<<dim3((unsigned)k, CS_COUNTERS / 32), 1024, 0, stream>>>(
+            d_pt_tiles, k, (u32*)P[61], (u32*)P[62], (u32*)P[63], h->ctl);
+        L.stop();
+    }
     // ---- record chunks: from the counts (one synchronisation) or from the plan
     // Records of m >= 3 come in two key classes: levels whose node keys fit
     // 31 bits (class 1) are sorted and scanned with 32-bit keys, the others
@@ -742,7 +991,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         const u32* nmask = nullptr;                // planned: class-1 levels per instance (device)
     };
     std::vector<Chunk> chunks;
-    std::vector<u32> nlev(k), lvl, qlvl;
+    std::vector<u32> nlev(k), lvl, qlvl, ilvl, iqlvl;
     u64 T_flat = 0, T_shared = 0;  // flat-map records in all, and those k_group forms in shared memory
     auto level_bits = [&](int s, u32 lv) -> u32 {
         if (M == 1) return 0u;
@@ -787,6 +1036,11 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         cudaMemcpyAsync(h_lvl + (size_t)k * LMAX, qlvl_tot, sizeof(u32) * k * LMAX, cudaMemcpyDeviceToHost, stream);
         cudaMemcpyAsync(hp + rec_pos, rec_all, sizeof(unsigned long long) * k, cudaMemcpyDeviceToHost, stream);
         cudaMemcpyAsync(h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
+        u32* h_ilvl = (u32*)(hp + item_pos);
+        if (items) {
+            cudaMemcpyAsync(h_ilvl, P[62], sizeof(u32) * k * LMAX, cudaMemcpyDeviceToHost, stream);
+            cudaMemcpyAsync(h_ilvl + (size_t)k * LMAX, P[63], sizeof(u32) * k * LMAX, cudaMemcpyDeviceToHost, stream);
+        }
         L.stop();
         e = cudaStreamSynchronize(stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "point phase");
@@ -802,6 +1056,10 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         lvl.assign(h_lvl, h_lvl + (size_t)k * LMAX);
         qlvl.assign(h_lvl + (size_t)k * LMAX, h_lvl + (size_t)2 * k * LMAX);
         const unsigned long long* h_rec = (const unsigned long long*)(hp + rec_pos);
+        if (items) {
+            ilvl.assign(h_ilvl, h_ilvl + (size_t)k * LMAX);
+            iqlvl.assign(h_ilvl + (size_t)k * LMAX, h_ilvl + (size_t)2 * k * LMAX);
+        }
         for (int s = 0; s < k; ++s) {
             inst[s] = h_inst[s];
             nlev[s] = inst[s].nQ + inst[s].nD == 0 ? 0u : (M == 1 ? 1u : inst[s].b[0]);
@@ -956,6 +1214,18 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             k_top_carry<Op><<<dim3((unsigned)multi.size(), TOP_STRIDE / 32), 1024, 0, stream>>>(
                 d_multi, d_prange, d_inst, top_agg, (u32)nranges);
             L.stop();
+        }
+    }
+
+    // ---- m = 3: the first rank's levels above the groups, a problem of m = 2
+    // per node
+    ItemStage IS{};
+    if constexpr (M == 3) {
+        if (items) {
+            IS = ItemStage{k, &ilvl, &iqlvl, NC, d_chunk_off, d_pt_offs, d_pt_tiles, pr0, pr1, (u32*)P[59],
+                           (u32*)P[60], (u32*)P[61], d_inst, P[18]};
+            domagg_status st = run_items<Op>(h, L, inst, IS);
+            if (st) return st;
         }
     }
 
@@ -1190,7 +1460,9 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             L.start(KIND_REDUCE, (double)C.Tq * sizeof(Part) + (double)(qe - qb) * (8 + sizeof(typename Op::Out)));
             k_reduce<Op, M><<<grid, 256, 0, stream>>>(d_chunk_off, k, C.k0, C.k1, d_pt_offs, pr0, pr1, pr2, pj,
                                                       qchunk_base, d_pt_tiles, (const u32*)P[25], d_qsbase, d_inst,
-                                                      partial, (u32)C.Tq, gacc, govf);
+                                                      partial, (u32)C.Tq, gacc, govf, (const Part*)IS.part, IS.n_part,
+                                                      (const u32*)P[60], (const u32*)P[61],
+                                                      IS.qseg ? IS.qseg + (size_t)C.k0 * LMAX : nullptr);
             L.stop();
         }
         Tq_all += C.Tq;
@@ -1224,20 +1496,49 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
 
 typedef std::vector<PlannedChunk> Planned;
 
+// Where the items' line lies: from 2^20 points on the records they replace
+// outweigh the items' launches and two synchronisations (9e5 points with 12
+// rank bits: 1518 us by records, 1618 by items; 2e6 points: 5.0 ms by records,
+// 3.4 by items; 2^22: 12.0 and 7.8); above 2^25 points their workspace (about
+// 160 bytes per point and level) would be the larger one.  Not for planned
+// runs (the nodes' sizes are read back), capped or fixed workspaces, shards,
+// the basic variant, or a split of the flat map that is not the default one.
+bool items_allowed(const domagg_ctx* h, const std::vector<Inst>& inst, const Planned* pl) {
+    if (pl || h->no_alloc || h->max_ws || h->nodes == 0 || h->group_bits != GROUP_MAX_BITS) return false;
+    u64 n = 0;
+    for (const Inst& I : inst) {
+        if (I.nshards || I.out_lo || (I.flags >> 3)) return false;
+        n += (u64)I.nD + I.nQ;
+    }
+    return n <= (1ull << 25) && (h->nodes == 2 || n >= ITEM_MIN_POINTS);
+}
+
 template <int M, class Op>
 domagg_status run_ct(domagg_ctx* h, std::vector<Inst>& inst, domagg_dtype ct, bool negate, cudaStream_t s,
-                     const Planned* pl) {
+                     const Planned* pl, bool items) {
+    if constexpr (M == 3) {
+        if (items && items_allowed(h, inst, pl)) {
+            std::vector<Inst> I = inst;
+            const domagg_status st = ct == DOMAGG_F32 ? run<M, Op, true>(h, I, negate, s, nullptr, true)
+                                                      : run<M, Op, false>(h, I, negate, s, nullptr, true);
+            if (st != DOMAGG_ERR_OOM) {
+                inst.swap(I);
+                return st;
+            }
+            h->err.clear();  // too many nodes, or no room for the items: the records
+        }
+    }
     return ct == DOMAGG_F32 ? run<M, Op, true>(h, inst, negate, s, pl) : run<M, Op, false>(h, inst, negate, s, pl);
 }
 
 template <class Op>
 domagg_status run_m(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype ct, bool negate, cudaStream_t s,
-                    const Planned* pl) {
+                    const Planned* pl, bool items) {
     switch (m) {
-        case 1: return run_ct<1, Op>(h, inst, ct, negate, s, pl);
-        case 2: return run_ct<2, Op>(h, inst, ct, negate, s, pl);
-        case 3: return run_ct<3, Op>(h, inst, ct, negate, s, pl);
-        default: return run_ct<4, Op>(h, inst, ct, negate, s, pl);
+        case 1: return run_ct<1, Op>(h, inst, ct, negate, s, pl, items);
+        case 2: return run_ct<2, Op>(h, inst, ct, negate, s, pl, items);
+        case 3: return run_ct<3, Op>(h, inst, ct, negate, s, pl, items);
+        default: return run_ct<4, Op>(h, inst, ct, negate, s, pl, items);
     }
 }
 
@@ -1401,21 +1702,8 @@ domagg_status pairs_launch_all(domagg_ctx* h, const std::vector<Inst>* small, do
     if (st) return st;
     layout((char*)h->pairs.p, (u32*)h->st_pairs.p);
     if (!up.empty() && !h->frozen) {
-        if (h->h_pair_cap < up.size()) {
-            if (h->h_pair) {
-                cudaDeviceSynchronize();
-                cudaFreeHost(h->h_pair);
-            }
-            h->h_pair = nullptr;
-            h->h_pair_cap = 0;
-            const size_t want = std::max<size_t>(up.size() + up.size() / 2, 1 << 16);
-            if (cudaMallocHost(&h->h_pair, want) != cudaSuccess) {
-                cudaGetLastError();
-                h->h_pair = nullptr;
-                return fail(h, DOMAGG_ERR_OOM, "pinned memory for the tables");
-            }
-            h->h_pair_cap = want;
-        }
+        st = grow_pinned_tables(h, up.size());
+        if (st) return st;
         memcpy(h->h_pair, up.data(), up.size());
         cudaMemcpyAsync(h->pairs.p, h->h_pair, up.size(), cudaMemcpyHostToDevice, stream);
     }
@@ -1505,19 +1793,19 @@ domagg_status run_pairs_one(domagg_ctx* h, int m, const Inst& I, domagg_dtype ct
 }
 
 domagg_status dispatch(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype ct, domagg_dtype wt,
-                       domagg_op op, bool negate, cudaStream_t s, const Planned* pl = nullptr, bool pairs = true) {
+                       domagg_op op, bool negate, cudaStream_t s, const Planned* pl, bool pairs, bool items) {
     if (pairs && !pl && inst.size() == 1 && pairs_allowed(h, m, inst[0]) && pairs_fit(inst[0])) {
         const domagg_status st = run_pairs_one(h, m, inst[0], ct, wt, op, negate, s);
         if (st != DOMAGG_ERR_OOM) return st;
         h->err.clear();  // the pipeline may fit a capped workspace that the pairs' partials do not
     }
-    if (op == DOMAGG_COUNT) return run_m<OpCount>(h, m, inst, ct, negate, s, pl);
-    if (op == DOMAGG_SUM && wt == DOMAGG_F32) return run_m<OpSumF32>(h, m, inst, ct, negate, s, pl);
-    if (op == DOMAGG_SUM && wt == DOMAGG_I64) return run_m<OpSumI64>(h, m, inst, ct, negate, s, pl);
-    if (op == DOMAGG_MAX && wt == DOMAGG_I32) return run_m<OpMaxI32>(h, m, inst, ct, negate, s, pl);
-    if (op == DOMAGG_MAX && wt == DOMAGG_F32) return run_m<OpMaxF32>(h, m, inst, ct, negate, s, pl);
-    if (op == DOMAGG_MIN && wt == DOMAGG_I32) return run_m<OpMinI32>(h, m, inst, ct, negate, s, pl);
-    if (op == DOMAGG_MIN && wt == DOMAGG_F32) return run_m<OpMinF32>(h, m, inst, ct, negate, s, pl);
+    if (op == DOMAGG_COUNT) return run_m<OpCount>(h, m, inst, ct, negate, s, pl, items);
+    if (op == DOMAGG_SUM && wt == DOMAGG_F32) return run_m<OpSumF32>(h, m, inst, ct, negate, s, pl, items);
+    if (op == DOMAGG_SUM && wt == DOMAGG_I64) return run_m<OpSumI64>(h, m, inst, ct, negate, s, pl, items);
+    if (op == DOMAGG_MAX && wt == DOMAGG_I32) return run_m<OpMaxI32>(h, m, inst, ct, negate, s, pl, items);
+    if (op == DOMAGG_MAX && wt == DOMAGG_F32) return run_m<OpMaxF32>(h, m, inst, ct, negate, s, pl, items);
+    if (op == DOMAGG_MIN && wt == DOMAGG_I32) return run_m<OpMinI32>(h, m, inst, ct, negate, s, pl, items);
+    if (op == DOMAGG_MIN && wt == DOMAGG_F32) return run_m<OpMinF32>(h, m, inst, ct, negate, s, pl, items);
     return fail(h, DOMAGG_ERR_INVALID_ARG, "unsupported (op, weight dtype) pair");
 }
 
@@ -1599,6 +1887,9 @@ bool set_tuning(domagg_ctx* h, const std::string& name, int value) {
     } else if (name == "top_bits") {
         if (value < 0 || value > TOP_MAX_BITS) return false;
         h->top_bits = value;
+    } else if (name == "nodes") {
+        if (value < 0 || value > 2) return false;
+        h->nodes = value;
     } else if (name == "pairs") {
         if (value < 0 || value > 1) return false;
         h->use_pairs = value != 0;
@@ -1689,8 +1980,10 @@ domagg_status domagg_destroy(domagg_handle h) {
     if (!h) return DOMAGG_ERR_INVALID_ARG;
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
-    for (DevBuf* b : {&h->pts, &h->recs, &h->st_multi, &h->st_seg, &h->stage, &h->st_wv, &h->pairs, &h->st_pairs})
+    for (DevBuf* b : {&h->pts, &h->recs, &h->st_multi, &h->st_seg, &h->stage, &h->st_wv, &h->pairs, &h->st_pairs,
+                      &h->items})
         if (b->p) cudaFree(b->p);
+    if (h->sub) domagg_destroy(h->sub);
     if (h->ctl) cudaFree(h->ctl);
     if (h->h_pair) cudaFreeHost(h->h_pair);
     if (h->h_pin) cudaFreeHost(h->h_pin);
@@ -2081,7 +2374,7 @@ domagg_status plan_group(domagg_plan p, int m, const std::vector<Inst>& part, do
     p->groups.push_back(g);
     domagg_plan_s::Group& G = p->groups.back();
     std::vector<Inst> measured = part;
-    st = dispatch(G.ctx, m, measured, p->ct, p->wt, p->op, false, s, nullptr, false);
+    st = dispatch(G.ctx, m, measured, p->ct, p->wt, p->op, false, s, nullptr, false, false);
     if (st) return plan_fail(p, st, G.ctx->err);
     if (cudaStreamSynchronize(s) != cudaSuccess) return plan_fail(p, DOMAGG_ERR_CUDA, "measuring run");
     // capacity budget: 2^32 positions and ~60% of the free device memory
@@ -2421,7 +2714,13 @@ domagg_status domagg_timing_read(domagg_handle h, domagg_timing* out) {
     cudaSetDevice(h->device);
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(h, e, "timing");
-    for (const TimedLaunch& t : h->log) {
+    std::vector<TimedLaunch> log = h->log;
+    if (h->sub) {  // the nodes' launches
+        log.insert(log.end(), h->sub->log.begin(), h->sub->log.end());
+        h->sub->log.clear();
+        h->sub->pool_used = 0;
+    }
+    for (const TimedLaunch& t : log) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, t.a, t.b);
         if (t.kind < 0 || t.kind >= DOMAGG_TIMING_KINDS) continue;

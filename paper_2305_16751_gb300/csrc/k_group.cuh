@@ -66,7 +66,7 @@ __host__ __device__ constexpr size_t group_smem_bytes() {
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
-                                                    u32 cap, u32 avg, int max_bits, int top_bits) {
+                                                    u32 cap, u32 avg, int max_bits, int top_bits, int items) {
     __shared__ u32 s_ovf[32];
     __shared__ u32 s_done;
     const int s = blockIdx.x;
@@ -128,6 +128,10 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
                 if (lv >= tS) tmask |= 1u << lv;
                 else mask |= 1u << lv;
             }
+        if (M == 3 && items) {  // the levels above the groups by items (k_items.cuh)
+            tmask = mask;
+            mask = 0;
+        }
         I.tS = tS;
         I.topmask = n > 0 ? tmask : 0u;
         I.lvmask = n > 0 ? mask : 0u;

@@ -724,7 +724,11 @@ __global__ __launch_bounds__(256) void k_reduce(const u32* __restrict__ chunk_of
                                                 const Inst* __restrict__ inst,
                                                 const typename Op::Part* __restrict__ partial, u32 n_partial,
                                                 const typename Op::Part* __restrict__ gacc,
-                                                const unsigned char* __restrict__ govf) {
+                                                const unsigned char* __restrict__ govf,
+                                                const typename Op::Part* __restrict__ ipart, u32 n_ipart,
+                                                const u32* __restrict__ iqchunk_base,
+                                                const u32* __restrict__ itile_excl,
+                                                const u32* __restrict__ iqseg_base /*[k1-k0][LMAX]*/) {
     typedef typename Op::Part Part;
     __shared__ u32 s_mask[8][LMAX];  // per warp: query lanes holding a record of level lv
     __shared__ u32 s_base[8][LMAX];  // per warp: first partial slot of level lv in this chunk
@@ -802,6 +806,26 @@ __global__ __launch_bounds__(256) void k_reduce(const u32* __restrict__ chunk_of
                     for (u32 kk = 0; kk < c1 && base + kk < n_partial; ++kk)
                         acc = Op::F(acc, Op::from_part(partial[base + kk]));
                 }
+            }
+        }
+        if (M == 3 && ipart) {
+            // the levels taken by items: one partial per query and level, in
+            // slots as for m = 2
+            const u32 ibits = q ? pr0[p] & low_mask(I.b[0]) & I.topmask : 0u;
+            __syncwarp();
+            s_base[warp][lane] = __ldg(iqseg_base + (u64)(s - k0) * LMAX + lane) +
+                                 __ldg(iqchunk_base + (u64)c * LMAX + lane) +
+                                 __ldg(itile_excl + (u64)(__ldg(pt_tiles + s) + (c - __ldg(chunk_off + s)) / CS_CHUNKS) *
+                                                        CS_COUNTERS + LMAX + lane);
+            s_mask[warp][lane] = warp_transpose32(ibits, (u32)lane);
+            __syncwarp();
+            u32 rem = ibits;
+#pragma unroll 4
+            while (rem) {
+                const u32 lv = __ffs(rem) - 1;
+                rem &= rem - 1;
+                const u32 slot = s_base[warp][lv] + (u32)__popc(s_mask[warp][lv] & lt);
+                if (domagg_check(slot < n_ipart, SITE_REDUCE)) acc = Op::F(acc, Op::from_part(ipart[slot]));
             }
         }
         if (q) {
