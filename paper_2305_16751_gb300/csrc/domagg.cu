@@ -667,6 +667,11 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         const u64 want = (u64)TOP_RANGES_PER_SM * (u64)std::max(h->sms, 1);
         const u64 tiles = (N + TOP_TILE - 1) / TOP_TILE;
         range_pts = (u32)std::min<u64>(TOP_TILE * std::max<u64>(1, (tiles + want - 1) / want), 1ull << 30);
+        // fewer points than a tile per SM: smaller tiles, one per SM (not in a
+        // capped or fixed workspace: every range holds its nodes' F)
+        const u64 sm = (u64)std::max(h->sms, 1);
+        if (N < sm * TOP_TILE && !h->no_alloc && !h->max_ws)
+            range_pts = (u32)std::min<u64>(TOP_TILE, std::max<u64>(1, (N / sm + 1023) / 1024) * 1024);
         u64 nr = 0;
         for (int s = 0; s < k; ++s) {
             prange_off[s] = (u32)nr;
@@ -945,10 +950,12 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     }
     // ---- the levels whose records go through HBM (this shard's, and for
     // m = 2 the levels above the groups of ranks that k_group takes)
+    // points of a group on average, at most (one group per SM for few points)
+    const bool tight = h->no_alloc || h->max_ws > 0;
+    const u32 gavg = M == 3 ? g3_avg(N, tight) : group_avg(N, h->sms, h->top_bits == TOP_MAX_BITS && !tight);
     L.start(KIND_SMALL, 0.0);
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,
-                                            govf, M == 3 ? G3_CAP : GROUP_CAP,
-                                            M == 3 ? g3_avg(N, h->no_alloc || h->max_ws > 0) : 0xffffffffu,
+                                            govf, M == 3 ? G3_CAP : group_cap(gavg), gavg,
                                             use_groups ? h->group_bits : 0,
                                             use_top ? h->top_bits : 0, items ? 1 : 0);
     cudaMemsetAsync(rec_all, 0, sizeof(unsigned long long) * k, stream);
@@ -1141,6 +1148,40 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         }
     }
 
+    // ---- m = 2: the top levels per range of tiles in the order of the last
+    // coordinate (k_top), then the nodes' carries across the ranges; beside
+    // the groups, which they do not read from, on a stream of the handle: of
+    // few points either fills a part of the chip, of many the one's last CTAs
+    // run beside the other's first (8.38 -> 7.96 ms at 2^24 per side)
+    const bool top_beside = use_top && nranges > 0 && use_groups && h->overlap;
+    if (top_beside) {
+        cudaEventRecord(h->ev_fork, stream);
+        cudaStreamWaitEvent(h->aux[0], h->ev_fork, 0);
+        L.stream = h->aux[0];
+    }
+    if (use_top && nranges > 0) {
+        typedef typename Op::Acc Acc;
+        constexpr size_t tsm = TopSmem<Acc>::TOTAL;
+        if (!L.frozen) cudaFuncSetAttribute(k_top<Op, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm);
+        const int li = L.lookback_index();
+        L.start(KIND_TOP, (double)N * (4.0 + (WT == 3 ? 0.0 : sizeof(W))) +
+                              (double)NQ * sizeof(Acc) +
+                              (double)nranges * TOP_STRIDE * sizeof(Acc));
+        k_top<Op, WT><<<(unsigned)h->sms, TOP_THREADS, tsm, L.stream>>>(d_inst, k, d_prange, d_pt_offs, range_pts, pr0,
+                                                                      (const W*)P[18], topv, top_agg,
+                                                                      (u32)nranges, h->ctl, li);
+        L.stop();
+        if (!multi.empty()) {
+            L.start(KIND_SMALL, 0.0);
+            k_top_carry<Op><<<dim3((unsigned)multi.size(), TOP_STRIDE / 32), 1024, 0, L.stream>>>(
+                d_multi, d_prange, d_inst, top_agg, (u32)nranges);
+            L.stop();
+        }
+    }
+    if (top_beside) {
+        cudaEventRecord(h->ev_join[0], h->aux[0]);
+        L.stream = stream;
+    }
     // ---- a shard's group parts start at the unit (its group kernel writes
     // only its own groups' queries)
     if (use_groups && inst[0].nshards > 1 && N > 0) {
@@ -1182,7 +1223,8 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             if (!L.frozen) cudaFuncSetAttribute(k_group<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
             L.start(KIND_GROUP, (double)N * 8.0 + (double)NQ * sizeof(Part));
             k_group<Op><<<(unsigned)h->sms, GROUP_THREADS, gsm, stream>>>(d_inst, k, gslot, rstart, gval[0], gval[1],
-                                                                          (const W*)P[18], gacc, h->ctl, li);
+                                                                          (const W*)P[18], gacc, group_cap(gavg),
+                                                                          h->ctl, li);
             L.stop();
         } else {
             // m = 3: the group-sorted rank and position, the second rank and
@@ -1195,28 +1237,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             L.stop();
         }
     }
-    // ---- m = 2: the top levels per range of tiles in the order of the last
-    // coordinate (k_top), then the nodes' carries across the ranges
-    if (use_top && nranges > 0) {
-        typedef typename Op::Acc Acc;
-        constexpr size_t tsm = TopSmem<Acc>::TOTAL;
-        if (!L.frozen) cudaFuncSetAttribute(k_top<Op, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm);
-        const int li = L.lookback_index();
-        L.start(KIND_TOP, (double)N * (4.0 + (WT == 3 ? 0.0 : sizeof(W))) +
-                              (double)NQ * (sizeof(Acc) + (use_groups ? sizeof(Part) : 0.0)) +
-                              (double)nranges * TOP_STRIDE * sizeof(Acc));
-        k_top<Op, WT><<<(unsigned)h->sms, TOP_THREADS, tsm, stream>>>(d_inst, k, d_prange, d_pt_offs, range_pts, pr0,
-                                                                      (const W*)P[18], gacc, topv, top_agg,
-                                                                      (u32)nranges, h->ctl, li);
-        L.stop();
-        if (!multi.empty()) {
-            L.start(KIND_SMALL, 0.0);
-            k_top_carry<Op><<<dim3((unsigned)multi.size(), TOP_STRIDE / 32), 1024, 0, stream>>>(
-                d_multi, d_prange, d_inst, top_agg, (u32)nranges);
-            L.stop();
-        }
-    }
-
+    if (top_beside) cudaStreamWaitEvent(stream, h->ev_join[0], 0);
     // ---- m = 3: the first rank's levels above the groups, a problem of m = 2
     // per node
     ItemStage IS{};

@@ -41,6 +41,19 @@ constexpr int GROUP_ITEMS = 12;          // points per thread, at most
 constexpr u32 GROUP_CAP = GROUP_THREADS * GROUP_ITEMS;  // points per group in shared memory
 constexpr u32 GROUP_NODES = 1u << (GROUP_MAX_BITS - 1);  // nodes of one level in a group, at most
 
+// m = 2: points of a group on average, at most, in a call over N points: no
+// limit of its own from a full group per SM on, below that a group per SM
+// (the levels above them go to the top tiles, also one per SM and beside the
+// groups: a call of 1.7e5 points 390 -> 332 us).
+// A group above eight times that would keep one SM busy long after the others:
+// it overflows, as one that shared memory does not hold.
+__host__ __device__ constexpr u32 group_avg(u64 N, int sms, bool top) {
+    const u64 c = N / (u64)(sms > 0 ? sms : 1);
+    return !top || c >= GROUP_CAP ? 0xffffffffu : (c <= 1024u ? 1024u : (u32)c);
+}
+
+__host__ __device__ constexpr u32 group_cap(u32 avg) { return avg >= GROUP_CAP / 8u ? GROUP_CAP : 8u * avg; }
+
 template <typename Acc>
 __host__ __device__ constexpr size_t group_smem_bytes() {
     return (size_t)GROUP_CAP * sizeof(Acc) + (size_t)Padded<GROUP_CAP>::value * sizeof(u32) +
@@ -52,7 +65,10 @@ __host__ __device__ constexpr size_t group_smem_bytes() {
 // many for shared memory: heavy ties) hold at most a quarter of the points
 // and which hold at most `avg` points on average, and the number of groups G (m = 2: k_group; m = 3: k_group3); gS = 0 (no
 // level in groups) if no width qualifies, or if the instance takes another
-// path.  govf[pt_off + g] = 1 marks this shard's groups that overflow: their
+// path.  m = 2 prefers the widest without any group above `cap`, where the
+// levels from there up still fit the top tiles: overflowing groups' records
+// in HBM cost more than a level in the tiles (0.34 of 2.14 ms at 5.7e6 points
+// with a seventh of them in such groups).  govf[pt_off + g] = 1 marks this shard's groups that overflow: their
 // points' levels below gS go through the records in HBM.  With top_bits > 0, the
 // levels from tS = max(gS, b0 - top_bits) up go to k_top, and the levels
 // [gS, tS) through the records in HBM (lvmask); both masks hold this
@@ -68,7 +84,6 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
                                                     u32 cap, u32 avg, int max_bits, int top_bits, int items) {
     __shared__ u32 s_ovf[32];
-    __shared__ u32 s_done;
     const int s = blockIdx.x;
     Inst& I = inst[s];
     const u32 n = I.nD + I.nQ;
@@ -89,21 +104,20 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
             if (c > cap) ov += c;
         }
         for (int o = 16; o >= 1; o >>= 1) ov += __shfl_xor_sync(0xffffffffu, ov, o);
+        __syncthreads();
         if ((threadIdx.x & 31) == 0) s_ovf[threadIdx.x >> 5] = ov;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            u32 t = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_ovf[w];
-            s_done = (t <= n / 4u && n <= (u64)avg * g_n) ? 1u : 0u;
-        }
-        __syncthreads();
-        const bool ok = s_done != 0u;
-        __syncthreads();
-        if (ok) {
-            chosen = (u32)S;
-            G = g_n;
-            break;
-        }
+        ov = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) ov += s_ovf[w];
+        const bool ok = ov <= n / 4u && n <= (u64)avg * g_n;
+        if (ok && (!chosen || ov == 0u)) chosen = (u32)S;
+        // m = 2: on to a narrower width without overflow, as long as the
+        // levels above it fit the top tiles
+        const bool narrower = M == 2 && top_bits > 0 && S > 1 && b0 - (u32)(S - 1) <= (u32)top_bits;
+        if (chosen && (ov == 0u || !narrower)) break;
+    }
+    if (chosen) {
+        G = (Uu + (1u << (chosen - ns)) - 1u) >> (chosen - ns);
     }
     if (chosen && govf) {  // this shard's groups that overflow
         const u32 us = chosen - ns, nsh = max(I.nshards, 1u);
@@ -412,7 +426,7 @@ __global__ __launch_bounds__(GROUP_THREADS, 1) void k_group(const Inst* __restri
                                                             const u32* __restrict__ rstart, const u64* __restrict__ gv0,
                                                             const u64* __restrict__ gv1,
                                                             const typename Op::W* __restrict__ pw,
-                                                            typename Op::Part* __restrict__ gacc, Ctl* ctl,
+                                                            typename Op::Part* __restrict__ gacc, u32 cap, Ctl* ctl,
                                                             int launch_idx) {
     typedef typename Op::Acc Acc;
     typedef GScan<Acc> E;
@@ -440,7 +454,7 @@ __global__ __launch_bounds__(GROUP_THREADS, 1) void k_group(const Inst* __restri
         const u32 a = __ldg(rs + (g << us)), e = __ldg(rs + min((g + 1u) << us, Uu));
         const bool odd = ((I.b[0] - gS + RADIX_BITS - 1) / RADIX_BITS) & 1u;
         const u64* __restrict__ gv = (odd ? gv1 : gv0) + I.pt_off + a;
-        if (e - a > GROUP_CAP) {  // too large for shared memory: its levels go through HBM
+        if (e - a > cap) {  // too large (cap <= GROUP_CAP, as in k_group_plan): its levels go through HBM
             group_unit_parts<Op>(gv, e - a, I, gacc);
             __syncthreads();
             continue;

@@ -12,8 +12,7 @@
 // order, instructions 6m+1 .. 6m+3).  A node's records continue across
 // tiles and ranges, so the scan carries, per node, F over the node's data in
 // the range's earlier tiles (frun, in shared memory), and every query keeps
-// F over its partial results of the range's top levels and of the levels
-// below gS (those from k_group, by position: gacc) in topv.  What the
+// F over its partial results of the range's top levels in topv.  What the
 // range's nodes gathered (agg) is then scanned across the ranges of the
 // instance in a fixed order (k_top_carry), and the per-query reduction adds
 // to each query, for every top level where it has a record, the carry of its
@@ -68,11 +67,9 @@ __device__ __forceinline__ TopRange top_range(u32 r, const u32* prange_off, int 
 
 // The top levels of every range (see the file comment).  Persistent CTAs
 // (one per SM) take ranges from a counter.  Inputs, in the order of the last
-// coordinate: pr0 (rank | QUERY_BIT), pw (a datum's weight bits, or its
-// 8-byte weight for WT = 1) and, for an instance with groups, gacc (a
-// query's F over the levels below gS).  Writes topv[x] (queries: F over
-// their partial results of the range's top levels and the levels below gS,
-// the unit if none) and agg[r][h] (F over the range's data of node h, heap
+// coordinate: pr0 (rank | QUERY_BIT) and pw (a datum's weight bits, or its
+// 8-byte weight for WT = 1).  Writes topv[x] (queries: F over their partial
+// results of the range's top levels, the unit if none) and agg[r][h] (F over the range's data of node h, heap
 // order; rows r < nrows, the rows the caller reserved: a range outside them
 // is skipped).
 template <class Op, int WT>
@@ -81,7 +78,6 @@ __global__ __launch_bounds__(TOP_THREADS, 1) void k_top(const Inst* __restrict__
                                                         const u32* __restrict__ pt_offs, u32 range_pts,
                                                         const u32* __restrict__ pr0,
                                                         const typename Op::W* __restrict__ pw,
-                                                        const typename Op::Part* __restrict__ gacc,
                                                         typename Op::Acc* __restrict__ topv,
                                                         typename Op::Acc* __restrict__ agg, u32 nrows, Ctl* ctl,
                                                         int launch_idx) {
@@ -112,7 +108,6 @@ __global__ __launch_bounds__(TOP_THREADS, 1) void k_top(const Inst* __restrict__
         const TopRange R = top_range(r, prange_off, k, pt_offs, range_pts);
         const Inst& I = inst[R.s];
         const u32 tmask = I.topmask, tS = I.tS, b0 = I.b[0];
-        const bool grouped = I.gS != 0u;
         // (the instance's levels from tS up: nb <= TOP_MAX_BITS by k_group_plan)
         const u32 nb = tmask ? b0 - tS : 0u;
         if (nb > 0u && DOMAGG_GUARD(nb <= (u32)TOP_MAX_BITS, SITE_GROUP_NODE)) {
@@ -141,7 +136,7 @@ __global__ __launch_bounds__(TOP_THREADS, 1) void k_top(const Inst* __restrict__
                         const bool q = (v[kk] & QUERY_BIT) != 0u;
                         w[kk] = Op::e();
                         if (i < n) {
-                            if (q) w[kk] = grouped ? Op::from_part(gacc[a0 + i]) : Op::e();
+                            if (q) w[kk] = Op::e();
                             else if constexpr (Op::GATHER) w[kk] = Op::from_w(pw[a0 + i]);
                             else if constexpr (WT == 3) w[kk] = Op::from_pay(0u);
                             else w[kk] = Op::from_pay((typename Op::Pay)pw[a0 + i]);
@@ -231,8 +226,8 @@ __global__ __launch_bounds__(1024) void k_top_carry(const u32* __restrict__ mult
 
 // Per-query reduction of m = 2 with top levels (replaces k_reduce there):
 // one block of TOP_RED_THREADS per range of the chunk's instances [k0, k1).
-// For each query: F over topv (the range's top levels and the levels below
-// gS; gacc alone for an instance without top levels), its partials of the
+// For each query: F over topv (the range's top levels), gacc (the levels
+// below gS), its partials of the
 // levels that went through the records in HBM (slots as in k_reduce) and,
 // for every top level where it has a record, the carry of its node from the
 // instance's earlier ranges (staged in shared memory).
@@ -288,7 +283,8 @@ __global__ __launch_bounds__(TOP_RED_THREADS) void k_reduce_top(int k, int k0, c
         }
         if (__ballot_sync(0xffffffffu, q) == 0u) continue;
         Acc acc = Op::e();
-        if (q) acc = tmask ? topv[p] : (I.gS ? Op::from_part(gacc[p]) : Op::e());
+        if (q && tmask) acc = topv[p];
+        if (q && I.gS) acc = Op::F(acc, Op::from_part(gacc[p]));
         const u32 rec = q ? bits0 & hbm_levels(I, a, govf) : 0u;
         if (__ballot_sync(0xffffffffu, rec != 0u)) {  // levels whose records went through HBM: their partials
             if ((u32)lane < b0)
