@@ -26,9 +26,10 @@
  *     never frees caller memory.
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream).  Device
  *     entry points enqueue work on it.  domagg_forward and domagg_backward
- *     synchronise the stream once in mid-call (they read the record count to
- *     size their workspace) and return with the rest of the work enqueued;
- *     outputs are valid once the stream has been synchronised.
+ *     synchronise the stream once in the call (they read the record count to
+ *     size their workspace, or the device's error bits; large calls of m = 3
+ *     read their nodes' sizes as well) and return with the rest of the work
+ *     enqueued; outputs are valid once the stream has been synchronised.
  *   - Supported (op, weight dtype) -> output dtype:
  *       SUM   int64 -> int64 (wraps modulo 2^64), float32 -> float32
  *       MAX   int32 -> int32, float32 -> float32

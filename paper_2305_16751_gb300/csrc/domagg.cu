@@ -26,6 +26,7 @@
 #include "k_records.cuh"
 #include "k_top.cuh"
 #include "k_wavelet.cuh"
+#include "k_line.cuh"
 #include "k_pairs.cuh"
 
 using namespace domagg;
@@ -947,6 +948,52 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     if (inst[0].flags & FLAG_WAVELET) {
         if constexpr (M <= 2) return run_wavelet<M, Op>(h, inst, d_inst, perm, r0, N, L, stream, hp, ctl_pos);
         else return fail(h, DOMAGG_ERR_UNSUPPORTED, "the level-wise formulation takes m <= 2");
+    }
+    // ---- m = 1: the scan of F over the permutation itself (k_line.cuh; a
+    // shard takes the records)
+    if constexpr (M == 1) {
+        if (inst[0].nshards == 0) {
+            typedef typename Op::Acc Acc;
+            Acc* tagg = (Acc*)P[25];
+            constexpr size_t lsm = line_smem<Op, WT>();
+            if (!L.frozen)
+                cudaFuncSetAttribute(k_line_apply<Op, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
+            const double wb = WT == 3 ? 0.0 : sizeof(W);
+            L.start(KIND_COUNT_SCAN, (double)N * 4 + (double)(N - NQ) * 2 * wb);
+            k_line_sum<Op, WT><<<(unsigned)ntp, LINE_THREADS, 0, stream>>>(perm, d_pt_offs, d_pt_tiles, k, d_inst,
+                                                                          (W*)P[18], tagg);
+            L.stop();
+            L.start(KIND_SMALL, 0.0);
+            k_line_carry<Op><<<(unsigned)k, 1024, 0, stream>>>(d_pt_tiles, tagg);
+            L.stop();
+            L.start(KIND_SEGSCAN, (double)N * (4 + wb) + (double)NQ * sizeof(typename Op::Out));
+            k_line_apply<Op, WT><<<(unsigned)ntp, LINE_THREADS, lsm, stream>>>(perm, d_pt_offs, d_pt_tiles, k, d_inst,
+                                                                              (const W*)P[18], tagg);
+            L.stop();
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_fail(h, e, "launch");
+            if (planned) return DOMAGG_OK;
+            Ctl* h_ctl = (Ctl*)(hp + ctl_pos);
+            L.start(KIND_D2H, 0.0);
+            cudaMemcpyAsync(h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
+            L.stop();
+            e = cudaStreamSynchronize(stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "point phase");
+            if (const u32 site = bounds_site(true)) return bounds_error(h, site);
+            h->ctl_host = *h_ctl;
+            if (h_ctl->error) {
+                const u32 bits = h_ctl->error;
+                cudaMemsetAsync(&h->ctl->error, 0, sizeof(u32), stream);
+                cudaStreamSynchronize(stream);
+                return device_error(h, bits);
+            }
+            memset(&h->stats, 0, sizeof(h->stats));
+            h->stats.n_points = h->stats.n_records = (int64_t)N;  // a record per point, none of them written
+            h->stats.n_query_records = (int64_t)NQ;
+            h->stats.m = 1;
+            h->stats.workspace_bytes = (int64_t)h->held();
+            return DOMAGG_OK;
+        }
     }
     // ---- the levels whose records go through HBM (this shard's, and for
     // m = 2 the levels above the groups of ranks that k_group takes)
