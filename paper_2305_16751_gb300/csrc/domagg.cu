@@ -684,11 +684,16 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     }
     const u64 nranges = prange_off[k];
 
+    // one block, at the same offsets on the device and in the pinned area: the
+    // record counts (per level, of queries, per instance) and the instance
+    // table, read back in one copy; the table and the offsets, uploaded in one
+    const size_t lvl_bytes = 2 * sizeof(u32) * k * LMAX + sizeof(unsigned long long) * k;
+    const size_t off_bytes = 3 * sizeof(u32) * (k + 1) + (use_top ? sizeof(u32) * (2 * k + 2) : 0);
+    const size_t up_bytes = sizeof(Inst) * k + off_bytes;
+
     // ---- point workspace
     auto carve_points = [&](Carver& c, void** P) {
-        P[0] = c.take<Inst>(k);
-        P[1] = c.take<u32>(k + 1);  // pt_offs
-        P[2] = c.take<u32>(k + 1);  // q_offs
+        P[0] = c.take<char>(lvl_bytes + up_bytes);
         P[3] = c.take<u32>(k + 1);  // point tiles
         P[4] = c.take<u32>(N);      // rk0
         P[5] = c.take<u32>(M >= 3 ? N : 0);  // rk1
@@ -701,15 +706,12 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         P[12] = c.take<u32>(M >= 2 ? N : 0);  // pr0
         P[13] = c.take<u32>(M >= 3 ? N : 0);  // pr1
         P[14] = c.take<u32>(N);     // pj
-        P[15] = c.take<u32>(k + 1);  // chunk offsets
         P[16] = c.take<u32>((size_t)NC * LMAX);  // query chunk bases per level
-        P[17] = c.take<u32>((size_t)k * LMAX);   // query records per (instance, level)
         P[18] = c.take<W>(WT == 3 ? 0 : N);  // weights in the order of the last coordinate
         P[19] = c.take<u32>((size_t)k * 4 * RADIX);  // hist
         P[20] = c.take<u32>((size_t)k * 4 * RADIX);  // digit offsets
         P[21] = c.take<u32>(k + 1);                  // the sorts' tile map
         P[22] = c.take<u32>((size_t)NC * LMAX);      // chunk bases per level
-        P[23] = c.take<u32>((size_t)k * LMAX);       // records per (instance, level)
         P[24] = c.take<u32>((size_t)sort_range_bound(pt_sizes) * RADIX);  // first-pass range bases
         P[25] = c.take<u32>((size_t)ntp * CS_COUNTERS);                   // per point tile: rank / flat-map counts
         P[26] = c.take<u32>(M >= 4 ? N : 0);  // rk2
@@ -740,20 +742,15 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         P[50] = c.take<u32>(grp ? k : 0);        // group-id bits per instance
         P[51] = c.take<u32>(grp ? k + 1 : 0);    // group slot offsets
         // m = 2 top levels: per query F over its range's top levels, per range
-        // F of every top-level node (then the carries), the range table, the
-        // instances of several ranges
+        // F of every top-level node (then the carries)
         P[52] = c.take<typename Op::Acc>(use_top ? N : 0);
         P[53] = c.take<typename Op::Acc>(use_top ? (size_t)nranges * TOP_STRIDE : 0);
-        P[54] = c.take<u32>(use_top ? k + 1 : 0);
-        P[55] = c.take<u32>(use_top ? std::max<size_t>(multi.size(), 1) : 0);
         // groups: per query (by position in the order of the last
         // coordinate) F over the levels below gS
         P[56] = c.take<typename Op::Part>(grp ? N : 0);
         // groups: this call's groups too large for shared memory (a flag per
-        // group, at the instance's point offset); per instance, every
-        // record of the flat map (a statistic)
+        // group, at the instance's point offset)
         P[57] = c.take<unsigned char>(grp ? N : 0);
-        P[58] = c.take<unsigned long long>(k);
         // m = 3, the levels above the groups by items: their counts
         P[59] = c.take<u32>(items ? (size_t)NC * LMAX : 0);
         P[60] = c.take<u32>(items ? (size_t)NC * LMAX : 0);
@@ -770,24 +767,26 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         Carver c2(h->pts.p);
         carve_points(c2, P);
     }
-    Inst* d_inst = (Inst*)P[0];
-    u32 *d_pt_offs = (u32*)P[1], *d_q_offs = (u32*)P[2], *d_pt_tiles = (u32*)P[3];
+    u32 *lvl_tot = (u32*)P[0], *qlvl_tot = lvl_tot + (size_t)k * LMAX;
+    unsigned long long* rec_all = (unsigned long long*)(qlvl_tot + (size_t)k * LMAX);
+    Inst* d_inst = (Inst*)(rec_all + k);
+    u32 *d_pt_offs = (u32*)(d_inst + k), *d_chunk_off = d_pt_offs + 2 * (k + 1), *d_prange = d_chunk_off + k + 1,
+        *d_multi = d_prange + k + 1;
+    u32* d_pt_tiles = (u32*)P[3];
     u32 *rk0 = (u32*)P[4], *rk1 = (u32*)P[5], *lk = (u32*)P[6], *kalt = (u32*)P[7];
     u32 *vA = (u32*)P[8], *vB = (u32*)P[9], *r0 = (u32*)P[10], *r1 = (u32*)P[11];
-    u32 *pr0 = (u32*)P[12], *pr1 = (u32*)P[13], *pj = (u32*)P[14], *d_chunk_off = (u32*)P[15];
+    u32 *pr0 = (u32*)P[12], *pr1 = (u32*)P[13], *pj = (u32*)P[14];
     u32 *rk2 = (u32*)P[26], *r2 = (u32*)P[27], *pr2 = (u32*)P[28];
-    u32 *qchunk_base = (u32*)P[16], *qlvl_tot = (u32*)P[17];
+    u32* qchunk_base = (u32*)P[16];
     u32 *hist = (u32*)P[19], *digit_off = (u32*)P[20];
     u32* d_sort_tiles = (u32*)P[21];
-    u32 *chunk_base = (u32*)P[22], *lvl_tot = (u32*)P[23];
+    u32* chunk_base = (u32*)P[22];
     u32 *rstart = (u32*)P[45], *gkey[2] = {(u32*)P[46], (u32*)P[47]}, *gbits = (u32*)P[50], *gslot = (u32*)P[51];
     u64* gval[2] = {(u64*)P[48], (u64*)P[49]};
     typename Op::Acc* topv = (typename Op::Acc*)P[52];
     typename Op::Part* gacc = (typename Op::Part*)P[56];
     unsigned char* govf = use_groups ? (unsigned char*)P[57] : nullptr;
-    unsigned long long* rec_all = (unsigned long long*)P[58];
     typename Op::Acc* top_agg = (typename Op::Acc*)P[53];
-    u32 *d_prange = (u32*)P[54], *d_multi = (u32*)P[55];
 
     // status words: point tiles x 256 digits (the records sort grows it later)
     {
@@ -798,34 +797,23 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     }
 
     // ---- upload the instance table and offsets
-    const size_t up_bytes = sizeof(Inst) * k + 3 * sizeof(u32) * (k + 1) + (use_top ? sizeof(u32) * (2 * k + 2) : 0);
-    const size_t lvl_pos = (up_bytes + 63) & ~(size_t)63;                          // level totals (read back)
-    const size_t rec_pos = (lvl_pos + 2 * sizeof(u32) * k * LMAX + 63) & ~(size_t)63;  // records per instance (read back)
-    const size_t ctl_pos = (rec_pos + sizeof(unsigned long long) * k + 63) & ~(size_t)63;  // control block (read back)
-    const size_t item_pos = (ctl_pos + sizeof(Ctl) + 63) & ~(size_t)63;                    // item totals (read back)
+    const size_t ctl_pos = (lvl_bytes + up_bytes + 63) & ~(size_t)63;    // control block (read back)
+    const size_t item_pos = (ctl_pos + sizeof(Ctl) + 63) & ~(size_t)63;  // item totals (read back)
     char* hp = nullptr;
     if (!planned) {
         domagg_status st = grow_pinned(h, item_pos + (items ? 2 * sizeof(u32) * k * LMAX : 0) + 64);
         if (st) return st;
         hp = (char*)h->h_pin;
-        memcpy(hp, inst.data(), sizeof(Inst) * k);
-        memcpy(hp + sizeof(Inst) * k, pt_offs.data(), sizeof(u32) * (k + 1));
-        memcpy(hp + sizeof(Inst) * k + sizeof(u32) * (k + 1), q_offs.data(), sizeof(u32) * (k + 1));
-        memcpy(hp + sizeof(Inst) * k + 2 * sizeof(u32) * (k + 1), chunk_off.data(), sizeof(u32) * (k + 1));
-        cudaMemcpyAsync(d_inst, hp, sizeof(Inst) * k, cudaMemcpyHostToDevice, stream);
-        cudaMemcpyAsync(d_pt_offs, hp + sizeof(Inst) * k, sizeof(u32) * (k + 1), cudaMemcpyHostToDevice, stream);
-        cudaMemcpyAsync(d_q_offs, hp + sizeof(Inst) * k + sizeof(u32) * (k + 1), sizeof(u32) * (k + 1),
-                        cudaMemcpyHostToDevice, stream);
-        cudaMemcpyAsync(d_chunk_off, hp + sizeof(Inst) * k + 2 * sizeof(u32) * (k + 1), sizeof(u32) * (k + 1),
-                        cudaMemcpyHostToDevice, stream);
+        memcpy(hp + lvl_bytes, inst.data(), sizeof(Inst) * k);
+        u32* ho = (u32*)(hp + lvl_bytes + sizeof(Inst) * k);
+        memcpy(ho, pt_offs.data(), sizeof(u32) * (k + 1));
+        memcpy(ho + (k + 1), q_offs.data(), sizeof(u32) * (k + 1));
+        memcpy(ho + 2 * (k + 1), chunk_off.data(), sizeof(u32) * (k + 1));
         if (use_top) {  // (a planned run reuses the tables its measuring run uploaded)
-            u32* hr = (u32*)(hp + sizeof(Inst) * k + 3 * sizeof(u32) * (k + 1));
-            memcpy(hr, prange_off.data(), sizeof(u32) * (k + 1));
-            memcpy(hr + k + 1, multi.data(), sizeof(u32) * multi.size());
-            cudaMemcpyAsync(d_prange, hr, sizeof(u32) * (k + 1), cudaMemcpyHostToDevice, stream);
-            if (!multi.empty())
-                cudaMemcpyAsync(d_multi, hr + k + 1, sizeof(u32) * multi.size(), cudaMemcpyHostToDevice, stream);
+            memcpy(ho + 3 * (k + 1), prange_off.data(), sizeof(u32) * (k + 1));
+            memcpy(ho + 4 * (k + 1), multi.data(), sizeof(u32) * multi.size());
         }
+        cudaMemcpyAsync(d_inst, hp + lvl_bytes, up_bytes, cudaMemcpyHostToDevice, stream);
         maybe_reset_epochs(h, stream);
     }
 
@@ -841,12 +829,9 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     L.pool_used = &h->pool_used;
 
     L.start(KIND_SMALL, 0.0);
-    k_begin<<<1, 64, 0, stream>>>(h->ctl);
+    k_start<<<1, 1024, 0, stream>>>(h->ctl, d_pt_offs, k, POINT_TILE, d_pt_tiles);
     L.stop();
     h->epoch_mirror += MAX_LAUNCHES;
-    L.start(KIND_SMALL, 0.0);
-    k_make_tiles<<<1, 1024, 0, stream>>>(d_pt_offs, k, POINT_TILE, d_pt_tiles);
-    L.stop();
 
     // (m = 2, the nodes of m = 3: keys and permutation are given)
     const bool pre = M == 2 && h->pre_keys != nullptr;
@@ -1004,8 +989,8 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,
                                             govf, M == 3 ? G3_CAP : group_cap(gavg), gavg,
                                             use_groups ? h->group_bits : 0,
-                                            use_top ? h->top_bits : 0, items ? 1 : 0);
-    cudaMemsetAsync(rec_all, 0, sizeof(unsigned long long) * k, stream);
+                                            use_top ? h->top_bits : 0, items ? 1 : 0, rec_all,
+                                            use_groups && k == 1 ? gslot : nullptr);
     L.stop();
     // ---- count / offset scan of the flat map, per level
     {
@@ -1081,14 +1066,11 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         }
     } else {
         // the one synchronisation: record counts and device errors
-        Inst* h_inst = (Inst*)hp;
-        u32* h_lvl = (u32*)(hp + lvl_pos);
+        const u32* h_lvl = (const u32*)hp;
+        const Inst* h_inst = (const Inst*)(hp + lvl_bytes);
         Ctl* h_ctl = (Ctl*)(hp + ctl_pos);
         L.start(KIND_D2H, 0.0);
-        cudaMemcpyAsync(h_inst, d_inst, sizeof(Inst) * k, cudaMemcpyDeviceToHost, stream);
-        cudaMemcpyAsync(h_lvl, lvl_tot, sizeof(u32) * k * LMAX, cudaMemcpyDeviceToHost, stream);
-        cudaMemcpyAsync(h_lvl + (size_t)k * LMAX, qlvl_tot, sizeof(u32) * k * LMAX, cudaMemcpyDeviceToHost, stream);
-        cudaMemcpyAsync(hp + rec_pos, rec_all, sizeof(unsigned long long) * k, cudaMemcpyDeviceToHost, stream);
+        cudaMemcpyAsync(hp, lvl_tot, lvl_bytes + sizeof(Inst) * k, cudaMemcpyDeviceToHost, stream);
         cudaMemcpyAsync(h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream);
         u32* h_ilvl = (u32*)(hp + item_pos);
         if (items) {
@@ -1109,7 +1091,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         // per instance: its levels, their record counts and sort-key bits
         lvl.assign(h_lvl, h_lvl + (size_t)k * LMAX);
         qlvl.assign(h_lvl + (size_t)k * LMAX, h_lvl + (size_t)2 * k * LMAX);
-        const unsigned long long* h_rec = (const unsigned long long*)(hp + rec_pos);
+        const unsigned long long* h_rec = (const unsigned long long*)(h_lvl + (size_t)2 * k * LMAX);
         if (items) {
             ilvl.assign(h_ilvl, h_ilvl + (size_t)k * LMAX);
             iqlvl.assign(h_ilvl + (size_t)k * LMAX, h_ilvl + (size_t)2 * k * LMAX);
@@ -1260,9 +1242,11 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                      planned ? nullptr : &gb_host, N};
         sort_pairs<u32, u64>(L, gs, gkey, gval, false, gbits_max, 0xffffffffu, KIND_HIST_POINTS, KIND_SORT_GROUPS,
                              gbits, true);
-        L.start(KIND_SMALL, 0.0);
-        k_group_slots<<<1, 1024, 0, stream>>>(d_inst, k, gslot);
-        L.stop();
+        if (k > 1) {
+            L.start(KIND_SMALL, 0.0);
+            k_group_slots<<<1, 1024, 0, stream>>>(d_inst, k, gslot);
+            L.stop();
+        }
         typedef typename Op::Acc Acc;
         const int li = L.lookback_index();
         if constexpr (M == 2) {
@@ -1419,26 +1403,33 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         u32* keys1[2] = {(u32*)R[11], (u32*)R[12]};
         Pay* pays1[2] = {(Pay*)R[13], (Pay*)R[14]};
         Part* partial = (Part*)R[7];
-        if (!planned) {
+        // without records through HBM only the reduction is left (it reads no
+        // slot base then)
+        const bool records = planned || C.T > 0;
+        if (records && !planned) {
             cudaMemcpyAsync(d_up, hb, sizeof(u32) * chunk_upload_words(C), cudaMemcpyHostToDevice, stream);
             maybe_reset_epochs(h, stream);
         }
         // fresh epoch and tile counters for the record phase of this chunk
-        L.start(KIND_SMALL, 0.0);
-        k_begin<<<1, 64, 0, stream>>>(h->ctl);
-        L.stop();
-        h->epoch_mirror += MAX_LAUNCHES;
-        L.next_lookback = 0;
+        if (records) {
+            L.start(KIND_SMALL, 0.0);
+            k_begin<<<1, 64, 0, stream>>>(h->ctl);
+            L.stop();
+            h->epoch_mirror += MAX_LAUNCHES;
+            L.next_lookback = 0;
+        }
         if (planned) {
             L.start(KIND_SMALL, 0.0);
             k_layout<M><<<1, 1024, 0, stream>>>(d_inst, C.k0, lvl_tot, qlvl_tot, C.slot_map, (int)nseg, (int)nseg0,
                                                 C.T0, C.T1, C.Tq, d_so, d_sbits, d_sbase, d_qsbase, h->ctl);
             L.stop();
         }
-        L.start(KIND_SMALL, 0.0);
-        k_make_tiles<<<1, 1024, 0, stream>>>(d_so, (int)nseg0, SEG_TILE, d_stiles);
-        if (nseg1) k_make_tiles<<<1, 1024, 0, stream>>>(d_so1, (int)nseg1, SEG_TILE1, d_stiles1);
-        L.stop();
+        if (records) {
+            L.start(KIND_SMALL, 0.0);
+            k_make_tiles<<<1, 1024, 0, stream>>>(d_so, (int)nseg0, SEG_TILE, d_stiles);
+            if (nseg1) k_make_tiles<<<1, 1024, 0, stream>>>(d_so1, (int)nseg1, SEG_TILE1, d_stiles1);
+            L.stop();
+        }
 
         // flat map (6m+1), level by level
         const u64 nchunk = chunk_off[C.k1] - chunk_off[C.k0];

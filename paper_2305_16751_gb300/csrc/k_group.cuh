@@ -60,6 +60,12 @@ __host__ __device__ constexpr size_t group_smem_bytes() {
            2 * GROUP_NODES * sizeof(unsigned short);
 }
 
+// Groups g < G with g % nshards == shard.
+__device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
+    const u32 ns = max(nshards, 1u);
+    return shard < G ? (G - shard + ns - 1u) / ns : 0u;
+}
+
 // Per instance (one block each): the largest gS <= min(GROUP_MAX_BITS, b0)
 // whose groups of 2^gS ranks that hold more than `cap` points each (too
 // many for shared memory: heavy ties) hold at most a quarter of the points
@@ -82,7 +88,9 @@ __host__ __device__ constexpr size_t group_smem_bytes() {
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
-                                                    u32 cap, u32 avg, int max_bits, int top_bits, int items) {
+                                                    u32 cap, u32 avg, int max_bits, int top_bits, int items,
+                                                    unsigned long long* __restrict__ rec_all,
+                                                    u32* __restrict__ gslot_off) {
     __shared__ u32 s_ovf[32];
     const int s = blockIdx.x;
     Inst& I = inst[s];
@@ -129,6 +137,11 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
     if (threadIdx.x == 0) {
         I.gS = chosen;
         I.G = chosen ? G : 0u;
+        rec_all[s] = 0ull;  // (the count scan adds up)
+        if (gslot_off) {    // a single instance: its slots (else k_group_slots)
+            gslot_off[0] = 0u;
+            gslot_off[1] = chosen ? group_slots(I.shard, I.nshards, G) : 0u;
+        }
         if (gbits) gbits[s] = chosen ? b0 - chosen + (M == 3 ? 1u : 0u) : 0u;
         // the levels >= gS of this shard: from tS up per tile (k_top), below
         // tS through the records in HBM
@@ -164,10 +177,7 @@ static __global__ __launch_bounds__(1024) void k_group_slots(const Inst* __restr
     for (int base = 0; base < k; base += blockDim.x) {
         const int s = base + threadIdx.x;
         u32 v = 0;
-        if (s < k && inst[s].gS) {  // groups g with g % nshards == shard
-            const u32 ns = max(inst[s].nshards, 1u), sh = inst[s].shard, G = inst[s].G;
-            v = sh < G ? (G - sh + ns - 1) / ns : 0u;
-        }
+        if (s < k && inst[s].gS) v = group_slots(inst[s].shard, inst[s].nshards, inst[s].G);
         u32 inc = v;
         for (int o = 1; o < 32; o <<= 1) {
             const u32 x = __shfl_up_sync(0xffffffffu, inc, o);

@@ -7,7 +7,7 @@
 namespace domagg {
 
 // Pipeline start: advance the look-back epoch and clear the tile counters.
-static __global__ void k_begin(Ctl* ctl) {
+__device__ __forceinline__ void begin_block(Ctl* ctl) {
     if (threadIdx.x == 0) {
         if (ctl->epoch_base > EPOCH_MASK - 4u * MAX_LAUNCHES) atomicOr(&ctl->error, ERR_EPOCH);
         ctl->epoch_base += MAX_LAUNCHES;
@@ -17,6 +17,8 @@ static __global__ void k_begin(Ctl* ctl) {
     }
     for (int i = threadIdx.x; i < MAX_LAUNCHES; i += blockDim.x) ctl->tile_ctr[i] = 0;
 }
+
+static __global__ void k_begin(Ctl* ctl) { begin_block(ctl); }
 
 // Epoch guard of a replayed plan (no host in the loop to reset the epochs):
 // once the epoch counter comes within `margin` of its limit, the status words
@@ -54,8 +56,9 @@ static __global__ void k_selftest_wait(int which, const u64* status, Ctl* ctl) {
 // ceil(len(s') / tile), tile_off[nseg] = total.  One block.
 // With seg_bits, segments whose keys have at most `skip_upto` bits get no
 // tiles (a radix pass starting at that bit leaves them where they are).
-static __global__ void k_make_tiles(const u32* __restrict__ seg_off, int nseg, u32 tile, u32* __restrict__ tile_off,
-                                    const u32* __restrict__ seg_bits = nullptr, u32 skip_upto = 0) {
+__device__ __forceinline__ void make_tiles_block(const u32* __restrict__ seg_off, int nseg, u32 tile,
+                                                 u32* __restrict__ tile_off, const u32* __restrict__ seg_bits,
+                                                 u32 skip_upto) {
     __shared__ u32 carry;
     __shared__ u32 warp_sum[32];
     if (threadIdx.x == 0) carry = 0;
@@ -85,6 +88,23 @@ static __global__ void k_make_tiles(const u32* __restrict__ seg_off, int nseg, u
         __syncthreads();
     }
     if (threadIdx.x == 0) tile_off[nseg] = carry;
+}
+
+// (clears n_zero words of `zero` as well: the sort's histogram, where it is small)
+static __global__ __launch_bounds__(1024) void k_make_tiles(const u32* __restrict__ seg_off, int nseg, u32 tile,
+                                                            u32* __restrict__ tile_off,
+                                                            const u32* __restrict__ seg_bits = nullptr,
+                                                            u32 skip_upto = 0, u32* __restrict__ zero = nullptr,
+                                                            u32 n_zero = 0) {
+    for (u32 x = threadIdx.x; x < n_zero; x += blockDim.x) zero[x] = 0u;
+    make_tiles_block(seg_off, nseg, tile, tile_off, seg_bits, skip_upto);
+}
+
+// Pipeline start: k_begin and the point tiles.
+static __global__ __launch_bounds__(1024) void k_start(Ctl* ctl, const u32* __restrict__ seg_off, int nseg, u32 tile,
+                                                       u32* __restrict__ tile_off) {
+    begin_block(ctl);
+    make_tiles_block(seg_off, nseg, tile, tile_off, nullptr, 0u);
 }
 
 // Order-preserving 32-bit keys (Sec. 4, instructions 5i-4: S_i = the i-th

@@ -139,18 +139,50 @@ __global__ __launch_bounds__(256) void k_range_count(const K* __restrict__ keys,
 // digit): slice sums, an exclusive scan of them in shared memory, then the
 // running bases.  32 warps for few segments of many ranges, one for many
 // segments of few.
+// With hist (the first pass) the block first scans the segment's histograms
+// of all passes into digit_off, its 32 digits of each.
 template <int WARPS>
-__global__ __launch_bounds__(WARPS * 32) void k_range_bases(const u32* __restrict__ range_off,
-                                                            const u32* __restrict__ digit_off, int npass,
-                                                            u32* __restrict__ range_cnt) {
+__global__ __launch_bounds__(WARPS * 32) void k_range_bases(const u32* __restrict__ range_off, u32* digit_off,
+                                                            int npass, u32* __restrict__ range_cnt,
+                                                            const u32* __restrict__ hist,
+                                                            const u32* __restrict__ seg_off) {
     __shared__ u32 s_sum[WARPS][33];
+    __shared__ u32 s_d0[32];
     const int seg = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = blockIdx.y * 32 + lane;
     const u32 r0 = __ldg(range_off + seg), r1 = __ldg(range_off + seg + 1);
     const u32 n = r1 - r0, per = (n + WARPS - 1) / WARPS;
+    if (hist) {
+        const u32 base = __ldg(seg_off + seg);
+        for (int p = warp; p < npass; p += WARPS) {
+            const u32* h = hist + ((u64)seg * npass + p) * RADIX + lane * 8;
+            u32 v[8], sum = 0;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                v[e] = h[e];
+                sum += v[e];
+            }
+            u32 inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 x = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += x;
+            }
+            u32 ex = base + inc - sum;
+            if (lane / 4 == (int)blockIdx.y) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    digit_off[((u64)seg * npass + p) * RADIX + lane * 8 + e] = ex;
+                    if (p == 0) s_d0[(lane & 3) * 8 + e] = ex;
+                    ex += v[e];
+                }
+            }
+        }
+        __syncthreads();
+    }
     if (n == 0u) return;
     const u32 a = r0 + min(n, (u32)warp * per), b = r0 + min(n, (u32)(warp + 1) * per);
-    u32 run = __ldg(digit_off + (u64)seg * npass * RADIX + d);
+    u32 run = hist ? s_d0[lane] : digit_off[(u64)seg * npass * RADIX + d];
     if (WARPS > 1) {
         u32 sum = 0;
         for (u32 r = a; r < b; r += 16) {  // 16 loads in flight

@@ -39,10 +39,13 @@ static u64 resident_ctas(size_t smem) {
 #endif
 constexpr u64 RANGE_SCAN_MIN = DOMAGG_RANGE_SCAN_MIN;
 static void range_bases(Launcher& L, const SortSpace& sp, u64 nranges, int npass, int pass, u32* range_cnt) {
-    const u32* off = sp.digit_off + (size_t)pass * RADIX;
+    u32* off = sp.digit_off + (size_t)pass * RADIX;
+    const u32* hist = pass == 0 ? sp.hist : nullptr;
     const dim3 grid(sp.nseg, RADIX / 32);
-    if (nranges >= 64ull * sp.nseg) k_range_bases<32><<<grid, 32 * 32, 0, L.stream>>>(sp.tile_off, off, npass, range_cnt);
-    else k_range_bases<1><<<grid, 32, 0, L.stream>>>(sp.tile_off, off, npass, range_cnt);
+    if (nranges >= 64ull * sp.nseg)
+        k_range_bases<32><<<grid, 32 * 32, 0, L.stream>>>(sp.tile_off, off, npass, range_cnt, hist, sp.seg_off);
+    else
+        k_range_bases<1><<<grid, 32, 0, L.stream>>>(sp.tile_off, off, npass, range_cnt, hist, sp.seg_off);
 }
 
 template <typename K, typename V, bool IOTA, bool STABLE>
@@ -101,24 +104,22 @@ int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool io
     if (nranges == 0) return 0;
     // the first pass takes its range bases from the histogram (no count, no look-back)
     u32* range_base = (sp.range_scratch && nranges <= sp.range_scratch_ranges) ? sp.range_scratch : nullptr;
-    L.start(KIND_SMALL, 0.0);
-    k_make_tiles<<<1, 1024, 0, L.stream>>>(sp.seg_off, sp.nseg, range_items, sp.tile_off, seg_bits, 0u);
-    L.stop();
     const int hist_smem = 8 * npass * RADIX * (int)sizeof(u32);  // per-warp histograms of every pass
-    const size_t hist_bytes = (size_t)sp.nseg * npass * RADIX * sizeof(u32);
-    cudaMemsetAsync(sp.hist, 0, hist_bytes, L.stream);
+    const size_t hist_words = (size_t)sp.nseg * npass * RADIX;
+    const bool clear = hist_words <= 65536;  // by the tile map's one block
+    L.start(KIND_SMALL, 0.0);
+    k_make_tiles<<<1, 1024, 0, L.stream>>>(sp.seg_off, sp.nseg, range_items, sp.tile_off, seg_bits, 0u, sp.hist,
+                                           clear ? (u32)hist_words : 0u);
+    L.stop();
+    if (!clear) cudaMemsetAsync(sp.hist, 0, hist_words * sizeof(u32), L.stream);
     L.start(kind_hist, sp.n_items * sizeof(K));
     k_radix_hist<K><<<(unsigned)nranges, 256, hist_smem, L.stream>>>(
         keys[0], sp.seg_off, sp.tile_off, sp.nseg, range_items, npass, 0, keymask, sp.hist, range_base, seg_bits);
     L.stop();
     L.start(KIND_SMALL, 0.0);
-    k_radix_offsets<<<sp.nseg * npass, RADIX, 0, L.stream>>>(sp.hist, sp.seg_off, npass, sp.digit_off);
+    if (range_base) range_bases(L, sp, nranges, npass, 0, range_base);
+    else k_radix_offsets<<<sp.nseg * npass, RADIX, 0, L.stream>>>(sp.hist, sp.seg_off, npass, sp.digit_off);
     L.stop();
-    if (range_base) {
-        L.start(KIND_SMALL, 0.0);
-        range_bases(L, sp, nranges, npass, 0, range_base);
-        L.stop();
-    }
     int cur = 0;
     for (int p = 0; p < npass; ++p) {
         if (p > 0 && seg_bits) {  // this pass's own ranges
