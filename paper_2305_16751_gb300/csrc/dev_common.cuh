@@ -76,6 +76,7 @@ struct Inst {
     // shard and the groups g with g % nshards == shard (host-filled; 0 of 1
     // for a whole forward)
     u32 lvmask, shard, nshards;
+    u32 has_hbm;  // any record of this call may go through HBM (lvmask, or a group of this shard overflows)
     float* out_lo;  // float32 sums of a shard: the low halves of the float-float partials (or null)
 };
 // The last of the M coordinates is not stored but constant (the basic

@@ -879,9 +879,15 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         k_tile_exscan<<<(unsigned)k, 1024, 0, C.stream>>>(d_pt_tiles, k, C.tile_cnt);
         L.stop();
         // the rank scatter in windows of destinations (each about 48 MB of
-        // ranks, so the L2 holds a window while its sectors fill)
+        // ranks, so the L2 holds a window while its sectors fill); instances
+        // that fit one window need none: a tile scatters into its own
+        // (40e6 points in 8e3 nodes, four windows: 1.0 -> 0.3 ms)
+        u64 most = 0;
+        for (u64 n : pt_sizes) most = std::max(most, n);
         const u64 nwin = h->rank_windows > 0 ? (u64)h->rank_windows
-                                             : std::max<u64>(1, (N * sizeof(u32) + (48ull << 20) - 1) / (48ull << 20));
+                         : most * sizeof(u32) <= (48ull << 20)
+                             ? 1
+                             : std::max<u64>(1, (N * sizeof(u32) + (48ull << 20) - 1) / (48ull << 20));
         const u64 span = (N + nwin - 1) / nwin;
         for (u64 w = 0; w < nwin; ++w) {
             const u64 lo = w * span, hi = std::min<u64>(N, lo + span);

@@ -127,13 +127,17 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
     if (chosen) {
         G = (Uu + (1u << (chosen - ns)) - 1u) >> (chosen - ns);
     }
+    u32 over = 0;
     if (chosen && govf) {  // this shard's groups that overflow
         const u32 us = chosen - ns, nsh = max(I.nshards, 1u);
         for (u32 g = threadIdx.x; g < G; g += blockDim.x) {
             const u32 lo = g << us, hi = min((g + 1u) << us, Uu);
-            govf[I.pt_off + g] = (__ldg(rs + hi) - __ldg(rs + lo) > cap && g % nsh == I.shard) ? 1u : 0u;
+            const u32 o = (__ldg(rs + hi) - __ldg(rs + lo) > cap && g % nsh == I.shard) ? 1u : 0u;
+            govf[I.pt_off + g] = (unsigned char)o;
+            over |= o;
         }
     }
+    over = (u32)__syncthreads_or((int)over);
     if (threadIdx.x == 0) {
         I.gS = chosen;
         I.G = chosen ? G : 0u;
@@ -162,6 +166,7 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
         I.tS = tS;
         I.topmask = n > 0 ? tmask : 0u;
         I.lvmask = n > 0 ? mask : 0u;
+        I.has_hbm = (I.lvmask || over) ? 1u : 0u;
     }
 }
 

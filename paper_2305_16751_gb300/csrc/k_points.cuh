@@ -500,7 +500,8 @@ __global__ __launch_bounds__(256) void k_count_scan(
             }
         }
         u32 mine = 0, mine_q = 0;
-        if (M <= 2) {
+        if (!I.has_hbm) {  // no record to place
+        } else if (M <= 2) {
             // one record per level: lane lv counts the lanes with bit lv set
             mine = (u32)__popc(warp_transpose32(hb, (u32)lane));
             mine_q = (u32)__popc(warp_transpose32(q ? hb : 0u, (u32)lane));
@@ -545,6 +546,7 @@ __global__ __launch_bounds__(256) void k_count_scan(
     const u32 base_q = s_w[warp][LMAX + lane];
     const u32 cbase = __ldg(chunk_off + L.seg) + (wstart - L.seg_begin) / 32u;
     u32 ra = 0, rq = 0;
+    if (!I.has_hbm) return;  // (the flat map and the reduction read no base then)
 #pragma unroll
     for (int i = 0; i < CS_ROUNDS; ++i) {
         if (wstart + (u32)i * 32u < L.end && (u32)lane < nlev) {
