@@ -19,9 +19,10 @@
 // 4096 ranks (5e3 points at 2^21 per side) cost 640 pairs per point against
 // the 13-14 second-rank level walks at each of 12 first-rank levels that did
 // the same in shared memory before (one CTA per group: 2.4 ms at 2^21 per
-// side and 0.6 ms for a single group of 8e3 points; now @NOW@).  A wider group
-// would double the pairs and save one level of records in HBM (0.25 ns per
-// point), about what it costs.
+// side and 0.6 ms for a single group of 8e3 points; by pairs 1.3 ms and
+// 0.06).  A wider group would double the pairs and save one level above
+// (k_items.cuh, or records in HBM), about what it costs; narrower ones
+// measured slower (2^21 per side 7.6 ms; groups of half the width 8.5).
 #pragma once
 #include "k_group.cuh"
 #include "k_pairs.cuh"
@@ -104,11 +105,11 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_group3(const Inst* __restri
         // a datum counts if every key is at most the query's bound
         u32 bound[PAIR_QPT][3];
         u32 dead = 0;
-        Acc acc[PAIR_QPT];
+        PairQueries<Op, 3> acc;
+        acc.clear();
 #pragma unroll
         for (int j = 0; j < PAIR_QPT; ++j) {
             const u32 q = tile * G3_QT + (u32)j * PAIR_LANES + ln;
-            acc[j] = Op::e();
             u32 r = 0, x = 0, r1 = 0;
             if (q < nq) {
                 const u64 v = gq[q];
@@ -144,16 +145,14 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_group3(const Inst* __restri
                 const uint4 t = *reinterpret_cast<const uint4*>(s_k[x]);
                 const u32 kd[3] = {t.x, t.y, t.z};
                 const Acc v = s_v[x];
-#pragma unroll
-                for (int j = 0; j < PAIR_QPT; ++j) PairAcc<Op, 3>::add(acc[j], kd, bound[j], v);
+                acc.add(kd, bound, v);
             }
-#pragma unroll
-            for (int j = 0; j < PAIR_QPT; ++j) acc[j] = Op::F(acc[j], Op::e());  // float-float: renormalised per stage
+            acc.settle();
         }
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < PAIR_QPT; ++j)
-            s_join[grp][(u32)j * PAIR_LANES + ln] = (dead >> j) & 1u ? Op::e() : acc[j];
+            s_join[grp][(u32)j * PAIR_LANES + ln] = (dead >> j) & 1u ? Op::e() : acc.get(j);
         __syncthreads();
         const u32 q = tile * G3_QT + tid;
         if (q < nq) {

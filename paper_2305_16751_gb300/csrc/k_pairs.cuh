@@ -91,14 +91,6 @@ __device__ __forceinline__ float pair_select_f32(const u32 (&k)[M], const u32 (&
             : "r"(k[0]), "r"(b[0]), "r"(k[1]), "r"(b[1]), "r"(k[2]), "r"(b[2]), "r"(k[3]), "r"(b[3]), C(v))
 
 template <int M>
-struct PairAcc<OpSumF32, M> {  // the exact error of every addition goes to the low part
-    static __device__ __forceinline__ void add(ff& a, const u32 (&k)[M], const u32 (&b)[M], ff v) {
-        const ff s = ff_two_sum(a.hi, pair_select_f32<M>(k, b, v.hi));
-        a.hi = s.hi;
-        a.lo = __fadd_rn(a.lo, s.lo);
-    }
-};
-template <int M>
 struct PairAcc<OpSumI64, M> {
     static __device__ __forceinline__ void add(long long& a, const u32 (&k)[M], const u32 (&b)[M], long long v) {
         DOMAGG_PAIR_STEP("add.s64", "l", a, v);
@@ -136,6 +128,77 @@ struct PairAcc<OpCount, M> {
     }
 };
 #undef DOMAGG_PAIR_STEP
+
+// The running F of a thread's PAIR_QPT queries.
+template <class Op, int M>
+struct PairQueries {
+    typename Op::Acc a[PAIR_QPT];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int j = 0; j < PAIR_QPT; ++j) a[j] = Op::e();
+    }
+    __device__ __forceinline__ void add(const u32 (&k)[M], const u32 (&b)[PAIR_QPT][M], typename Op::Acc v) {
+#pragma unroll
+        for (int j = 0; j < PAIR_QPT; ++j) PairAcc<Op, M>::add(a[j], k, b[j], v);
+    }
+    __device__ __forceinline__ void settle() {}
+    __device__ __forceinline__ typename Op::Acc get(int j) const { return a[j]; }
+};
+// Float-float sums take two queries per instruction (add.rn.f32x2: the same
+// roundings, half the issue slots of the seven additions: 13.3 -> 9.1 instructions per pair
+// for m = 2; then the half-rate compares and the two additions' lanes bind:
+// 192 planned problems 241 -> 226 us).  The exact
+// error of every addition goes to the low part; settle() renormalises.
+__device__ __forceinline__ u64 f2_pack(float x, float y) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(u64 v, float& x, float& y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ u64 f2_add(u64 x, u64 y) {
+    u64 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    return r;
+}
+__device__ __forceinline__ u64 f2_sub(u64 x, u64 y) {
+    u64 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    return r;
+}
+template <int M>
+struct PairQueries<OpSumF32, M> {
+    static_assert(PAIR_QPT % 2 == 0, "two queries per instruction");
+    u64 hi[PAIR_QPT / 2], lo[PAIR_QPT / 2];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int j = 0; j < PAIR_QPT / 2; ++j) hi[j] = lo[j] = 0ull;
+    }
+    __device__ __forceinline__ void add(const u32 (&k)[M], const u32 (&b)[PAIR_QPT][M], ff v) {
+#pragma unroll
+        for (int j = 0; j < PAIR_QPT / 2; ++j) {
+            const u64 x = f2_pack(pair_select_f32<M>(k, b[2 * j], v.hi), pair_select_f32<M>(k, b[2 * j + 1], v.hi));
+            const u64 h = hi[j], t = f2_add(h, x), z = f2_sub(t, h);  // Knuth's TwoSum, as ff_two_sum
+            lo[j] = f2_add(lo[j], f2_add(f2_sub(h, f2_sub(t, z)), f2_sub(x, z)));
+            hi[j] = t;
+        }
+    }
+    __device__ __forceinline__ ff get(int j) const {
+        float h[2], l[2];
+        f2_unpack(hi[j / 2], h[0], h[1]);
+        f2_unpack(lo[j / 2], l[0], l[1]);
+        return {h[j % 2], l[j % 2]};
+    }
+    __device__ __forceinline__ void settle() {
+#pragma unroll
+        for (int j = 0; j < PAIR_QPT / 2; ++j) {
+            const ff x = ff_add(get(2 * j), ff{0.f, 0.f}), y = ff_add(get(2 * j + 1), ff{0.f, 0.f});
+            hi[j] = f2_pack(x.hi, y.hi);
+            lo[j] = f2_pack(x.lo, y.lo);
+        }
+    }
+};
 
 // A partial another block wrote (through the L2).
 template <typename Acc>
@@ -187,11 +250,11 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_pairs(const __grid_constant
     // Strictly below key 0 there is nothing: such a query is dead (its F is e).
     u32 bound[PAIR_QPT][M];
     u32 dead = 0;
-    Acc acc[PAIR_QPT];
+    PairQueries<Op, M> acc;
+    acc.clear();
 #pragma unroll
     for (int j = 0; j < PAIR_QPT; ++j) {
         const u32 q = tile * PAIR_QT + (u32)j * PAIR_LANES + ln;
-        acc[j] = Op::e();
 #pragma unroll
         for (int i = 0; i < M; ++i) {
             u32 key = 0;
@@ -227,17 +290,15 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_pairs(const __grid_constant
                 if constexpr (M == 4) kd[3] = t.w;
             }
             const Acc v = s_v[x];
-#pragma unroll
-            for (int j = 0; j < PAIR_QPT; ++j) PairAcc<Op, M>::add(acc[j], kd, bound[j], v);
+            acc.add(kd, bound, v);
         }
-#pragma unroll
-        for (int j = 0; j < PAIR_QPT; ++j) acc[j] = Op::F(acc[j], Op::e());  // float-float: renormalised per stage
+        acc.settle();
     }
     if (nan) atomicOr(&C.ctl->error, ERR_NAN);
     // join the groups: from here on a thread holds one query
 #pragma unroll
     for (int j = 0; j < PAIR_QPT; ++j)
-        s_join[grp][(u32)j * PAIR_LANES + ln] = (dead >> j) & 1u ? Op::e() : acc[j];
+        s_join[grp][(u32)j * PAIR_LANES + ln] = (dead >> j) & 1u ? Op::e() : acc.get(j);
     __syncthreads();
     const u32 q = tile * PAIR_QT + tid;
     Acc r = s_join[0][tid];
