@@ -433,7 +433,7 @@ domagg_status grow_pinned_tables(domagg_ctx* h, size_t bytes) {
 // m = 3: what the items' stage reads of the point phase, and what it leaves:
 // a partial per (level, query item), at qseg[instance][level] + the query's
 // place in the level.
-constexpr u64 ITEM_MAX_NODES = 1u << 17, ITEM_MIN_POINTS = 1u << 20;
+constexpr u64 ITEM_MAX_NODES = 1u << 17, ITEM_MIN_POINTS = 1u << 19;
 struct ItemStage {
     int k;
     const std::vector<u32>*lvl, *qlvl;  // items and query items per (instance, level)
@@ -1256,12 +1256,25 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         typedef typename Op::Acc Acc;
         const int li = L.lookback_index();
         if constexpr (M == 2) {
-            constexpr size_t gsm = group_smem_bytes<Acc>();
-            if (!L.frozen) cudaFuncSetAttribute(k_group<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
+            constexpr size_t gsm = group_smem_bytes<Acc, GROUP_THREADS>();
+            constexpr size_t ssm = group_smem_bytes<Acc, GROUP_SMALL_THREADS>();
+            if (!L.frozen) {
+                cudaFuncSetAttribute(k_group<Op, GROUP_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
+                cudaFuncSetAttribute(k_group<Op, GROUP_SMALL_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)ssm);
+            }
+            // small groups, as far as the host knows, by the small kind
+            bool small = planned != nullptr;
+            for (int s = 0; s < k && !planned; ++s)
+                small = small || (inst[s].G && pt_sizes[s] <= (u64)GROUP_SMALL * inst[s].G);
             L.start(KIND_GROUP, (double)N * 8.0 + (double)NQ * sizeof(Part));
-            k_group<Op><<<(unsigned)h->sms, GROUP_THREADS, gsm, stream>>>(d_inst, k, gslot, rstart, gval[0], gval[1],
-                                                                          (const W*)P[18], gacc, group_cap(gavg),
-                                                                          h->ctl, li);
+            if (small)
+                k_group<Op, GROUP_SMALL_THREADS><<<4u * (unsigned)h->sms, GROUP_SMALL_THREADS, ssm, stream>>>(
+                    d_inst, k, gslot, rstart, gval[0], gval[1], (const W*)P[18], gacc, group_cap(gavg), 0u, h->ctl,
+                    L.lookback_index());
+            k_group<Op, GROUP_THREADS><<<(unsigned)h->sms, GROUP_THREADS, gsm, stream>>>(
+                d_inst, k, gslot, rstart, gval[0], gval[1], (const W*)P[18], gacc, group_cap(gavg),
+                small ? GROUP_SMALL : 0u, h->ctl, li);
             L.stop();
         } else {
             // m = 3: the group-sorted rank and position, the second rank and
@@ -1561,13 +1574,13 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
 
 typedef std::vector<PlannedChunk> Planned;
 
-// Where the items' line lies: from 2^20 points on the records they replace
-// outweigh the items' launches and two synchronisations (9e5 points with 12
-// rank bits: 1518 us by records, 1618 by items; 2e6 points: 5.0 ms by records,
-// 3.4 by items; 2^22: 12.0 and 7.8); above 2^25 points their workspace (about
-// 160 bytes per point and level) would be the larger one.  Not for planned
-// runs (the nodes' sizes are read back), capped or fixed workspaces, shards,
-// the basic variant, or a split of the flat map that is not the default one.
+// Where the items' line lies: from 2^19 points on the records they replace
+// outweigh the items' launches and two synchronisations (2e5 points: 653 us by
+// records, 818 by items; 6e5: 1598 and 1322; 9e5 with 12 rank bits: 1484 and
+// 1426; 2^22: 12.0 ms and 7.6); above 2^25 points their workspace (about 160
+// bytes per point and level) would be the larger one.  Not for planned runs
+// (the nodes' sizes are read back), capped or fixed workspaces, shards, the
+// basic variant, or a split of the flat map that is not the default one.
 bool items_allowed(const domagg_ctx* h, const std::vector<Inst>& inst, const Planned* pl) {
     if (pl || h->no_alloc || h->max_ws || h->nodes == 0 || h->group_bits != GROUP_MAX_BITS) return false;
     u64 n = 0;

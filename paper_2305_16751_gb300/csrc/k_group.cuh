@@ -54,9 +54,15 @@ __host__ __device__ constexpr u32 group_avg(u64 N, int sms, bool top) {
 
 __host__ __device__ constexpr u32 group_cap(u32 avg) { return avg >= GROUP_CAP / 8u ? GROUP_CAP : 8u * avg; }
 
-template <typename Acc>
+// k_group runs with 1024 threads, one block per SM, or, for groups of at most
+// GROUP_SMALL points, with 256, four per SM: a small group's levels are
+// barriers and block scans rather than points (a call of 1.7e5 points, groups
+// of 1e3: k_group 60 -> 43 us beside k_top, the call 286 -> 268).
+constexpr int GROUP_SMALL_THREADS = 256;
+constexpr u32 GROUP_SMALL = GROUP_SMALL_THREADS * GROUP_ITEMS;
+template <typename Acc, int T>
 __host__ __device__ constexpr size_t group_smem_bytes() {
-    return (size_t)GROUP_CAP * sizeof(Acc) + (size_t)Padded<GROUP_CAP>::value * sizeof(u32) +
+    return (size_t)T * GROUP_ITEMS * sizeof(Acc) + (size_t)Padded<T * GROUP_ITEMS>::value * sizeof(u32) +
            2 * GROUP_NODES * sizeof(unsigned short);
 }
 
@@ -360,8 +366,8 @@ __device__ __forceinline__ void group_levels(u32 n, u32 nb, u32 scan_mask, typen
         if (lane == 0) lex = ident;
         if (lane == 31) s_w[warp] = inc;
         __syncthreads();
-        if (warp == 0) {  // one warp scans the 32 warp totals (exclusive, in place)
-            E wi = s_w[lane];
+        if (warp == 0) {  // one warp scans the warps' totals (exclusive, in place)
+            E wi = lane < (int)(blockDim.x >> 5) ? s_w[lane] : ident;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const E nb = gscan_shfl_up(wi, o);
@@ -369,7 +375,7 @@ __device__ __forceinline__ void group_levels(u32 n, u32 nb, u32 scan_mask, typen
             }
             E wx = gscan_shfl_up(wi, 1);
             if (lane == 0) wx = ident;
-            s_w[lane] = wx;
+            s_w[lane] = wx;  // (32 entries, whatever the number of warps)
         }
         __syncthreads();
         const E ex = gscan_combine<Op>(s_w[warp], lex);
@@ -426,8 +432,10 @@ __device__ __forceinline__ void group_unit_parts(const u64* __restrict__ gv, u32
     }
 }
 
-// The deep levels of every group (see the file comment).  Persistent CTAs
-// (one per SM) take groups from a counter.  Inputs: the group-sorted points
+// The deep levels of every group of more than `above` points (see the file
+// comment).  Persistent CTAs (one per SM, or four of the small kind, which
+// leaves groups of more than its capacity to the other) take groups from a
+// counter.  Inputs: the group-sorted points
 // gv (per instance in buffer gv0 or gv1, by the parity of the group sort's
 // passes): (rank | QUERY_BIT) << 32 | payload, the payload being a query's
 // position x in the order of the last coordinate, a datum's weight bits, or
@@ -435,23 +443,23 @@ __device__ __forceinline__ void group_unit_parts(const u64* __restrict__ gv, u32
 // query's partial results of the levels below gS, as a partial (rounded once,
 // like a level's partial; read in that order by k_top and the per-query
 // reduction).
-template <class Op>
-__global__ __launch_bounds__(GROUP_THREADS, 1) void k_group(const Inst* __restrict__ inst, int k,
+template <class Op, int T>
+__global__ __launch_bounds__(T, T == GROUP_THREADS ? 1 : 4) void k_group(const Inst* __restrict__ inst, int k,
                                                             const u32* __restrict__ gslot_off,
                                                             const u32* __restrict__ rstart, const u64* __restrict__ gv0,
                                                             const u64* __restrict__ gv1,
                                                             const typename Op::W* __restrict__ pw,
-                                                            typename Op::Part* __restrict__ gacc, u32 cap, Ctl* ctl,
-                                                            int launch_idx) {
+                                                            typename Op::Part* __restrict__ gacc, u32 cap, u32 above,
+                                                            Ctl* ctl, int launch_idx) {
     typedef typename Op::Acc Acc;
     typedef GScan<Acc> E;
-    constexpr int T = GROUP_THREADS;
+    constexpr u32 CAP = (u32)T * GROUP_ITEMS;
     extern __shared__ __align__(128) unsigned char smem[];
     Acc* val = reinterpret_cast<Acc*>(smem);                              // by original index
-    u32* xh = reinterpret_cast<u32*>(smem + (size_t)GROUP_CAP * sizeof(Acc));  // handles, padded
-    unsigned short* nstart = reinterpret_cast<unsigned short*>(xh + Padded<GROUP_CAP>::value);
+    u32* xh = reinterpret_cast<u32*>(smem + (size_t)CAP * sizeof(Acc));  // handles, padded
+    unsigned short* nstart = reinterpret_cast<unsigned short*>(xh + Padded<CAP>::value);
     unsigned short* nzero = nstart + GROUP_NODES;
-    __shared__ E s_w[T / 32];
+    __shared__ E s_w[32];
     __shared__ u32 s_slot;
     const int tid = threadIdx.x;
     const u32 total = __ldg(gslot_off + k);
@@ -470,11 +478,15 @@ __global__ __launch_bounds__(GROUP_THREADS, 1) void k_group(const Inst* __restri
         const bool odd = ((I.b[0] - gS + RADIX_BITS - 1) / RADIX_BITS) & 1u;
         const u64* __restrict__ gv = (odd ? gv1 : gv0) + I.pt_off + a;
         if (e - a > cap) {  // too large (cap <= GROUP_CAP, as in k_group_plan): its levels go through HBM
-            group_unit_parts<Op>(gv, e - a, I, gacc);
+            if (T == GROUP_THREADS) group_unit_parts<Op>(gv, e - a, I, gacc);
             __syncthreads();
             continue;
         }
         const u32 n = e - a;
+        if (n <= above || n > CAP) {  // the other kind's
+            __syncthreads();
+            continue;
+        }
         const u32 lrmask = (1u << gS) - 1u;
         // the group's points in the order of the last coordinate: handles
         // (rank bits below gS | query bit | original index) and values
