@@ -230,18 +230,6 @@ __device__ __forceinline__ u32 match_digit8(u32 d, u32 valid) {
     return m;
 }
 
-// Adds one count for digit d (if valid) to a per-warp histogram h.  Lanes that
-// share lane 0's digit are added together (one atomic), which removes the
-// contention of skewed digit distributions where one digit dominates; the
-// other lanes add one each.
-__device__ __forceinline__ void warp_hist_add(u32* h, u32 d, bool valid, u32 lane) {
-    const u32 d0 = __shfl_sync(0xffffffffu, d, 0);
-    const bool same = valid && d == d0;
-    const u32 grp = __ballot_sync(0xffffffffu, same);
-    if (valid && !same) atomicAdd(&h[d], 1u);
-    else if (same && lane == (u32)(__ffs(grp) - 1)) atomicAdd(&h[d0], (u32)__popc(grp));
-}
-
 // Transpose of the warp's 32x32 bit matrix (lane l holds row l): returns the
 // lane's column, whose bit k is bit `lane` of lane k's row.  Five rounds that
 // swap off-diagonal blocks of 16, 8, 4, 2, 1 bits.
@@ -289,25 +277,15 @@ __device__ __forceinline__ u32 low_mask(u32 b) { return b >= 32 ? 0xffffffffu : 
 __device__ __forceinline__ u32 node_of(u32 r, u32 j) { return ((r >> j) | 1u) << j; }
 
 // ---------------------------------------------------------------------
-// TMA bulk copies into shared memory, completed on an mbarrier
+// mbarriers (a bounded wait; the self-test of the wait limits runs one out)
 // ---------------------------------------------------------------------
 __device__ __forceinline__ u32 smem_addr(const void* p) { return (u32)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(u64* bar, u32 count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-// Orders this thread's earlier generic-proxy shared-memory accesses before
-// later async-proxy (TMA) accesses to the same memory.
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive_expect_tx(u64* bar, u32 bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-// Global -> shared bulk copy; both addresses 16-byte aligned, bytes % 16 == 0.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, u32 bytes, u64* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
                  : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(u64* bar, u32 parity) {

@@ -2760,13 +2760,16 @@ domagg_status domagg_sync_status(domagg_handle h, void* stream) {
     cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sync");
     if (const u32 site = bounds_site(true)) return bounds_error(h, site);
-    u32 bits = 0;
-    e = cudaMemcpy(&bits, &h->ctl->error, sizeof(u32), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(h, e, "sync");
-    if (bits) {
-        cudaMemset(&h->ctl->error, 0, sizeof(u32));
-        cudaDeviceSynchronize();
-        return device_error(h, bits);
+    for (domagg_ctx* c : {h, h->sub}) {  // (the nodes' handle: m = 3)
+        if (!c) continue;
+        u32 bits = 0;
+        e = cudaMemcpy(&bits, &c->ctl->error, sizeof(u32), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(h, e, "sync");
+        if (bits) {
+            cudaMemset(&c->ctl->error, 0, sizeof(u32));
+            cudaDeviceSynchronize();
+            return device_error(h, bits);
+        }
     }
     return DOMAGG_OK;
 }
