@@ -13,7 +13,9 @@
 // themselves -- three compares, a select and F per pair (PairAcc), no node, no
 // split and no scan.
 //
-// Bound by instruction issue: 12 instructions per pair for a float-float sum.
+// Bound by instruction issue, on the half-rate pipe of the compares and the
+// select above all (issue active 64 %); a stage of data that lies wholly before
+// the tile's queries needs no third compare.
 // A group of c points costs c / 8 pairs per point (half of its points are
 // data, half queries, and a query meets the data before it only), so groups of
 // 4096 ranks (5e3 points at 2^21 per side) cost 640 pairs per point against
@@ -122,7 +124,8 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_group3(const Inst* __restri
             bound[j][1] = r1 - 1u;
             bound[j][2] = x - 1u;
         }
-        const u32 xmax = (u32)gq[min(nq, (tile + 1u) * G3_QT) - 1u];  // the tile's last query
+        // the tile's first and last query
+        const u32 xmin = (u32)gq[tile * G3_QT], xmax = (u32)gq[min(nq, (tile + 1u) * G3_QT) - 1u];
         for (u32 d0 = 0; d0 < nd; d0 += PAIR_STAGE) {
             const u32 m = min(PAIR_STAGE, nd - d0);
             __syncthreads();  // the previous stage is read
@@ -140,12 +143,20 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_group3(const Inst* __restri
             __syncthreads();
             if (s_k[0][2] > xmax) break;  // every datum from here on lies behind the tile's queries
             const u32 per = (m + PAIR_GROUPS - 1u) / PAIR_GROUPS, x1 = min(m, (grp + 1u) * per);
+            if (s_k[m - 1u][2] < xmin) {  // the whole stage lies before the tile: no position to compare
 #pragma unroll 4
-            for (u32 x = grp * per; x < x1; ++x) {
-                const uint4 t = *reinterpret_cast<const uint4*>(s_k[x]);
-                const u32 kd[3] = {t.x, t.y, t.z};
-                const Acc v = s_v[x];
-                acc.add(kd, bound, v);
+                for (u32 x = grp * per; x < x1; ++x) {
+                    const uint4 t = *reinterpret_cast<const uint4*>(s_k[x]);
+                    const u32 kd[3] = {t.x, t.y, t.z};
+                    acc.template add<2>(kd, bound, s_v[x]);
+                }
+            } else {
+#pragma unroll 4
+                for (u32 x = grp * per; x < x1; ++x) {
+                    const uint4 t = *reinterpret_cast<const uint4*>(s_k[x]);
+                    const u32 kd[3] = {t.x, t.y, t.z};
+                    acc.template add<3>(kd, bound, s_v[x]);
+                }
             }
             acc.settle();
         }

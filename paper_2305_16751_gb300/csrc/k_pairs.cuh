@@ -137,9 +137,19 @@ struct PairQueries {
 #pragma unroll
         for (int j = 0; j < PAIR_QPT; ++j) a[j] = Op::e();
     }
+    // a datum of keys k; the first C of them are compared
+    template <int C>
     __device__ __forceinline__ void add(const u32 (&k)[M], const u32 (&b)[PAIR_QPT][M], typename Op::Acc v) {
+        u32 kc[C];
 #pragma unroll
-        for (int j = 0; j < PAIR_QPT; ++j) PairAcc<Op, M>::add(a[j], k, b[j], v);
+        for (int i = 0; i < C; ++i) kc[i] = k[i];
+#pragma unroll
+        for (int j = 0; j < PAIR_QPT; ++j) {
+            u32 bc[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) bc[i] = b[j][i];
+            PairAcc<Op, C>::add(a[j], kc, bc, v);
+        }
     }
     __device__ __forceinline__ void settle() {}
     __device__ __forceinline__ typename Op::Acc get(int j) const { return a[j]; }
@@ -175,10 +185,20 @@ struct PairQueries<OpSumF32, M> {
 #pragma unroll
         for (int j = 0; j < PAIR_QPT / 2; ++j) hi[j] = lo[j] = 0ull;
     }
+    template <int C>
     __device__ __forceinline__ void add(const u32 (&k)[M], const u32 (&b)[PAIR_QPT][M], ff v) {
+        u32 kc[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) kc[i] = k[i];
 #pragma unroll
         for (int j = 0; j < PAIR_QPT / 2; ++j) {
-            const u64 x = f2_pack(pair_select_f32<M>(k, b[2 * j], v.hi), pair_select_f32<M>(k, b[2 * j + 1], v.hi));
+            u32 b0[C], b1[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                b0[i] = b[2 * j][i];
+                b1[i] = b[2 * j + 1][i];
+            }
+            const u64 x = f2_pack(pair_select_f32<C>(kc, b0, v.hi), pair_select_f32<C>(kc, b1, v.hi));
             const u64 h = hi[j], t = f2_add(h, x), z = f2_sub(t, h);  // Knuth's TwoSum, as ff_two_sum
             lo[j] = f2_add(lo[j], f2_add(f2_sub(h, f2_sub(t, z)), f2_sub(x, z)));
             hi[j] = t;
@@ -290,7 +310,7 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_pairs(const __grid_constant
                 if constexpr (M == 4) kd[3] = t.w;
             }
             const Acc v = s_v[x];
-            acc.add(kd, bound, v);
+            acc.template add<M>(kd, bound, v);
         }
         acc.settle();
     }
@@ -349,7 +369,9 @@ __global__ __launch_bounds__(PAIR_THREADS, 2) void k_pairs(const __grid_constant
 // problem takes eight blocks per coordinate (one block: 26 us at 8192 points,
 // 80 at 16000, 117 at 21000, longer than the pairs); a batch, whose
 // instances fill the chip, takes one.
-constexpr int PSTAT_THREADS = 1024;
+// Up to 8192 points a cluster's blocks have 256 threads (fewer warps whose
+// counts are scanned: 25 -> 22 us), else 1024.
+constexpr int PSTAT_THREADS = 1024, PSTAT_FEW_THREADS = 256;
 constexpr u32 PSTAT_CLUSTER = 8;                // blocks per coordinate of a single problem
 constexpr u32 PSTAT_MAX = 24u * PSTAT_THREADS;  // points of a problem, at most (24 registers of keys in one block)
 struct PairStatCall {
@@ -362,9 +384,9 @@ struct PairStatCall {
     int negate;
     Ctl* ctl;
 };
-template <int ITEMS>
+template <int ITEMS, int T>
 constexpr size_t pstat_smem() {  // two item buffers (keys, indices) and the warps' digit counts
-    return (size_t)PSTAT_THREADS * ITEMS * (ITEMS <= 16 ? 12 : 6) + (size_t)(PSTAT_THREADS / 32) * (RADIX + 1) * 4;
+    return (size_t)T * ITEMS * (ITEMS <= 16 ? 12 : 6) + (size_t)(T / 32) * (RADIX + 1) * 4;
 }
 __device__ __forceinline__ u32 cluster_rank() {
     u32 r;
@@ -392,10 +414,12 @@ __device__ __forceinline__ void cluster_st16(u32 a, unsigned short v) {
     asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory");
 }
 
-template <int M, bool F32, int ITEMS>
-__global__ __launch_bounds__(PSTAT_THREADS) void k_pair_stats(const __grid_constant__ PairStatCall C) {
+template <int M, bool F32, int ITEMS, int T>
+__global__ __launch_bounds__(T) void k_pair_stats(const __grid_constant__ PairStatCall C) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    constexpr int T = PSTAT_THREADS, W = T / 32, R = M - 1;
+    constexpr int W = T / 32, R = M - 1;
+    constexpr u32 PER = T / RADIX;  // threads per digit, eight warps' counts each
+    static_assert(PER * 8 == W && (PER == 1 || PER == 4), "digit scan");
     constexpr u32 CAP = (u32)T * ITEMS;  // items of a block
     // the items of the next digit go to the other buffer: no barrier between
     // a block's reads and its peers' next writes (with more than 16 items,
@@ -454,8 +478,7 @@ __global__ __launch_bounds__(PSTAT_THREADS) void k_pair_stats(const __grid_const
             pos[j] = (unsigned short)(__shfl_sync(0xffffffffu, old, leader) + (u32)__popc(peers & lt));
         }
         __syncthreads();
-        // four threads per digit take eight warps' counts each
-        const u32 d = (u32)tid >> 2, part = (u32)tid & 3u;
+        const u32 d = (u32)tid / PER, part = (u32)tid % PER;
         u32 c[8], sum = 0;
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
@@ -463,9 +486,12 @@ __global__ __launch_bounds__(PSTAT_THREADS) void k_pair_stats(const __grid_const
             sum += c[w];
         }
         // the block's count of the digit, to every block of the cluster
-        u32 quad = sum + __shfl_xor_sync(0xffffffffu, sum, 1);
-        quad += __shfl_xor_sync(0xffffffffu, quad, 2);
-        for (u32 r = part; r < size; r += 4u) cluster_st32(cluster_map(&s_ct[rank][d], r), quad);
+        u32 quad = sum;
+        if (PER == 4) {
+            quad += __shfl_xor_sync(0xffffffffu, quad, 1);
+            quad += __shfl_xor_sync(0xffffffffu, quad, 2);
+        }
+        for (u32 r = part; r < size; r += PER) cluster_st32(cluster_map(&s_ct[rank][d], r), quad);
         cluster_sync();
         // the digit's count over the blocks, and over those before this one
         u32 tot = 0, mine = 0;
@@ -474,7 +500,7 @@ __global__ __launch_bounds__(PSTAT_THREADS) void k_pair_stats(const __grid_const
             if (r < rank) mine += x;
             tot += x;
         }
-        u32 inc = part == 3u ? tot : 0u;  // over the digits, one thread of four
+        u32 inc = part == PER - 1u ? tot : 0u;  // over the digits, one thread of each
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const u32 x = __shfl_up_sync(0xffffffffu, inc, o);
@@ -488,14 +514,16 @@ __global__ __launch_bounds__(PSTAT_THREADS) void k_pair_stats(const __grid_const
             cluster_sync();  // s_ct read by all before it is written again
             continue;        // one digit for all: the order stays
         }
-        u32 before = inc - (part == 3u ? tot : 0u);  // digits below, of this warp (exact in the quad's last thread)
-        before = __shfl_sync(0xffffffffu, before, lane | 3);
+        u32 before = inc - (part == PER - 1u ? tot : 0u);  // digits below, of this warp (in the digit's last thread)
+        before = __shfl_sync(0xffffffffu, before, lane | (int)(PER - 1u));
         for (int w = 0; w < warp; ++w) before += s_tmp[w];
         u32 run = before + mine;
-        u32 pre = sum + __shfl_up_sync(0xffffffffu, sum, 1) * (part >= 1u ? 1u : 0u);
-        const u32 two = __shfl_up_sync(0xffffffffu, pre, 2);
-        if (part >= 2u) pre += two;
-        run += pre - sum;  // the digit's items in this block's warps before
+        if (PER == 4) {  // the digit's items in this block's warps before
+            u32 pre = sum + __shfl_up_sync(0xffffffffu, sum, 1) * (part >= 1u ? 1u : 0u);
+            const u32 two = __shfl_up_sync(0xffffffffu, pre, 2);
+            if (part >= 2u) pre += two;
+            run += pre - sum;
+        }
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
             s_wh[part * 8u + w][d] = run;

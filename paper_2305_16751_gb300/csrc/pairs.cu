@@ -18,13 +18,13 @@ static void launch_one(Launcher& L, const PairCall& C, unsigned blocks, bool bes
     cudaLaunchKernelEx(&cfg, k_pairs<M, Op, WT, F32>, C);
 }
 
-template <int M, bool F32, int ITEMS>
+template <int M, bool F32, int ITEMS, int T>
 static void launch_stats(Launcher& L, const PairStatCall& C, unsigned jobs, unsigned cluster) {
-    constexpr size_t smem = pstat_smem<ITEMS>();
-    cudaFuncSetAttribute(k_pair_stats<M, F32, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr size_t smem = pstat_smem<ITEMS, T>();
+    cudaFuncSetAttribute(k_pair_stats<M, F32, ITEMS, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(jobs * cluster);
-    cfg.blockDim = dim3(PSTAT_THREADS);
+    cfg.blockDim = dim3(T);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = L.stream;
     cudaLaunchAttribute at[1];
@@ -33,7 +33,7 @@ static void launch_stats(Launcher& L, const PairStatCall& C, unsigned jobs, unsi
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_pair_stats<M, F32, ITEMS>, C);
+    cudaLaunchKernelEx(&cfg, k_pair_stats<M, F32, ITEMS, T>, C);
 }
 
 template <int M, bool F32>
@@ -45,14 +45,14 @@ static void launch_mf(Launcher& L, PairOp op, const PairCall& C, unsigned blocks
             L.start(KIND_SMALL, 0.0);
             if (!st->tab) {  // a single problem: a cluster per coordinate
                 const unsigned cl = PSTAT_CLUSTER;
-                if (st_points <= 1u * cl * PSTAT_THREADS) launch_stats<M, F32, 1>(L, *st, st_jobs, cl);
-                else launch_stats<M, F32, 3>(L, *st, st_jobs, cl);
+                if (st_points <= 4u * cl * PSTAT_FEW_THREADS) launch_stats<M, F32, 4, PSTAT_FEW_THREADS>(L, *st, st_jobs, cl);
+                else launch_stats<M, F32, 3, PSTAT_THREADS>(L, *st, st_jobs, cl);
             } else if (st_points <= 2u * PSTAT_THREADS) {
-                launch_stats<M, F32, 2>(L, *st, st_jobs, 1);
+                launch_stats<M, F32, 2, PSTAT_THREADS>(L, *st, st_jobs, 1);
             } else if (st_points <= 8u * PSTAT_THREADS) {
-                launch_stats<M, F32, 8>(L, *st, st_jobs, 1);
+                launch_stats<M, F32, 8, PSTAT_THREADS>(L, *st, st_jobs, 1);
             } else {
-                launch_stats<M, F32, 24>(L, *st, st_jobs, 1);
+                launch_stats<M, F32, 24, PSTAT_THREADS>(L, *st, st_jobs, 1);
             }
             L.stop();
         }
