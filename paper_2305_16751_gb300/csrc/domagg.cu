@@ -433,7 +433,7 @@ domagg_status grow_pinned_tables(domagg_ctx* h, size_t bytes) {
 // m = 3: what the items' stage reads of the point phase, and what it leaves:
 // a partial per (level, query item), at qseg[instance][level] + the query's
 // place in the level.
-constexpr u64 ITEM_MAX_NODES = 1u << 17, ITEM_MIN_POINTS = 1u << 19;
+constexpr u64 ITEM_MAX_NODES = 1u << 17, ITEM_MIN_POINTS = 1u << 19, ITEM_MAX_POINTS = 1u << 25;
 struct ItemStage {
     int k;
     const std::vector<u32>*lvl, *qlvl;  // items and query items per (instance, level)
@@ -990,7 +990,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     // m = 2 the levels above the groups of ranks that k_group takes)
     // points of a group on average, at most (one group per SM for few points)
     const bool tight = h->no_alloc || h->max_ws > 0;
-    const u32 gavg = M == 3 ? g3_avg(N, tight) : group_avg(N, h->sms, h->top_bits == TOP_MAX_BITS && !tight);
+    const u32 gavg = M == 3 ? g3_avg(N, tight, items) : group_avg(N, h->sms, h->top_bits == TOP_MAX_BITS && !tight);
     L.start(KIND_SMALL, 0.0);
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,
                                             govf, M == 3 ? G3_CAP : group_cap(gavg), gavg,
@@ -1581,14 +1581,17 @@ typedef std::vector<PlannedChunk> Planned;
 // bytes per point and level) would be the larger one.  Not for planned runs
 // (the nodes' sizes are read back), capped or fixed workspaces, shards, the
 // basic variant, or a split of the flat map that is not the default one.
+bool items_handle(const domagg_ctx* h) {
+    return !h->no_alloc && !h->max_ws && h->nodes != 0 && h->group_bits == GROUP_MAX_BITS;
+}
 bool items_allowed(const domagg_ctx* h, const std::vector<Inst>& inst, const Planned* pl) {
-    if (pl || h->no_alloc || h->max_ws || h->nodes == 0 || h->group_bits != GROUP_MAX_BITS) return false;
+    if (pl || !items_handle(h)) return false;
     u64 n = 0;
     for (const Inst& I : inst) {
         if (I.nshards || I.out_lo || (I.flags >> 3)) return false;
         n += (u64)I.nD + I.nQ;
     }
-    return n <= (1ull << 25) && (h->nodes == 2 || n >= ITEM_MIN_POINTS);
+    return n <= ITEM_MAX_POINTS && (h->nodes == 2 || n >= ITEM_MIN_POINTS);
 }
 
 template <int M, class Op>
@@ -2338,17 +2341,32 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst, 
     domagg_status ret = DOMAGG_OK;
     for (int m = 1; m <= 4 && !ret; ++m) {
         if (groups[m].empty()) continue;
-        // one call per group of at most 2^31 - 1 points
+        // one call per group of at most 2^31 - 1 points (m = 3: as many as may
+        // go by items; the statistics are the group's)
+        const int64_t most = m == 3 && items_handle(h) ? (int64_t)ITEM_MAX_POINTS : ((int64_t)1 << 31) - 1;
         std::vector<Inst> part;
+        domagg_stats sum;
+        memset(&sum, 0, sizeof(sum));
         int64_t acc = 0;
+        int parts = 0;
         for (size_t i = 0; i <= groups[m].size() && !ret; ++i) {
-            const bool flush = i == groups[m].size() ||
-                               (acc + (int64_t)groups[m][i].nD + groups[m][i].nQ >= ((int64_t)1 << 31) - 1);
+            const bool flush = i == groups[m].size() || (acc + (int64_t)groups[m][i].nD + groups[m][i].nQ >= most);
             if (flush && !part.empty()) {
                 ret = dispatch(h, m, part, coord_dtype, weight_dtype, op, false, (cudaStream_t)stream, nullptr, false);
                 synced = true;
                 part.clear();
                 acc = 0;
+                domagg_stats& S = h->stats;
+                if (parts++) {
+                    S.n_points += sum.n_points;
+                    S.n_records += sum.n_records;
+                    S.n_query_records += sum.n_query_records;
+                    S.n_records_shared += sum.n_records_shared;
+                    S.record_key_bits = std::max(S.record_key_bits, sum.record_key_bits);
+                    S.record_passes = std::max(S.record_passes, sum.record_passes);
+                    for (int d = 0; d < 3; ++d) S.rank_bits[d] = 0, S.distinct[d] = 0;
+                }
+                sum = S;
             }
             if (i < groups[m].size()) {
                 part.push_back(groups[m][i]);

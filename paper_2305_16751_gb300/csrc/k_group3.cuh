@@ -41,9 +41,9 @@ constexpr u32 G3_CAP = 10240;
 // limit of its own (8192 ranks, a level of records less) where room for
 // records is short: a workspace that is capped or fixed, and calls that come
 // near the limit of 2^32 records.
-__host__ __device__ constexpr u32 g3_avg(u64 N, bool tight) {
+__host__ __device__ constexpr u32 g3_avg(u64 N, bool tight, bool items) {
     const u64 c = N / 64u;
-    if (tight || N > (1ull << 24)) return 0xffffffffu;
+    if (tight || (!items && N > (1ull << 24))) return 0xffffffffu;
     return c >= 7168u ? 7168u : (c <= 1024u ? 1024u : (u32)c);
 }
 
