@@ -159,8 +159,8 @@ u32 bounds_site_sort(bool clear);
 // With seg_bits (device, one entry per segment), segment s is sorted by its
 // first seg_bits[s] bits only and its result is in buffer
 // ceil(seg_bits[s] / 8) % 2; the return value is then meaningless.
-// stable = false allows any order among equal digits (for sorts whose result
-// is only the sorted key sequence).
+// stable = false allows any order among equal digits in the first pass of an
+// iota sort (for sorts whose result is only the sorted key sequence).
 template <typename K, typename V>
 int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool iota, int total_bits, K keymask,
                int kind_hist, int kind_pass, const u32* seg_bits = nullptr, bool stable = true);

@@ -74,7 +74,6 @@ int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool io
         cudaFuncSetAttribute(k_onesweep<K, V, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(k_onesweep<K, V, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(k_onesweep<K, V, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(k_onesweep<K, V, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(k_radix_hist<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_smem_max);
     }
     // ranges: about L.ranges_per_cta (4) per resident CTA, whole tiles, never
@@ -158,12 +157,13 @@ int sort_pairs(Launcher& L, const SortSpace& sp, K* keys[2], V* vals[2], bool io
         L.start(kind_pass, moved * (2.0 * sizeof(K) + vbytes));
         K *ki = keys[cur], *ko = keys[cur ^ 1];
         V *vi = vals[cur], *vo = vals[cur ^ 1];
+        // (only the first pass may leave equal digits in any order: a later one
+        // has to keep the order of the digits before it)
         if (iota && p == 0) {
             if (stable) launch_pass<K, V, true, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
             else launch_pass<K, V, true, false>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
         } else {
-            if (stable) launch_pass<K, V, false, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
-            else launch_pass<K, V, false, false>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
+            launch_pass<K, V, false, true>(L, grid, smem, ki, vi, ko, vo, sp, range_items, seg_bits, rb, npass, p, keymask, li);
         }
         L.stop();
         cur ^= 1;
