@@ -113,3 +113,25 @@ def test_nodes_float_sums_repeat_exactly():
     with knobs(nodes=0):
         ref = domagg.forward(Dd, Qd, wi, "sum").cpu().numpy()
     assert np.array_equal(got, ref)
+
+
+def test_batch_in_parts_equals_single_calls():
+    """More points of m = 3 than one call of the nodes takes (2^25): every
+    instance of the batch as its own call, bit for bit, and the statistics of
+    the whole."""
+    rng = np.random.default_rng(9500)
+    probs = []
+    for nD, nQ in ((7 << 20, 6 << 20), (4 << 20, 9 << 20), (300000, 1), (5 << 20, 5 << 20), (200000, 250000)):
+        D, Q, w = workloads.random_small(rng, 3, nD, nQ, 1 << 22, "i32", "i64")
+        probs.append((to_dev(D), to_dev(Q), to_dev(w)))
+    points = sum(p[0].shape[0] + p[1].shape[0] for p in probs)
+    assert points > 1 << 25
+    outs = domagg.batch(probs, "sum")
+    st = domagg.stats()
+    assert st["n_points"] == points
+    records = 0
+    for p, o in zip(probs, outs):
+        single = domagg.forward(*p, "sum")
+        assert torch().equal(o, single), tuple(p[0].shape)
+        records += domagg.stats()["n_records"]
+    assert st["n_records"] == records
