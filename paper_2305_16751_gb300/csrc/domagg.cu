@@ -1578,7 +1578,9 @@ typedef std::vector<PlannedChunk> Planned;
 // outweigh the items' launches and two synchronisations (2e5 points: 653 us by
 // records, 818 by items; 6e5: 1598 and 1322; 9e5 with 12 rank bits: 1484 and
 // 1426; 2^22: 12.0 ms and 7.6); above 2^25 points their workspace (about 160
-// bytes per point and level) would be the larger one.  Not for planned runs
+// bytes per point and level) would be the larger one, and a batch is cut into
+// parts of that size (2037 instances, 1.6e8 points: 164 ms; 272 as one call by
+// records).  Not for planned runs
 // (the nodes' sizes are read back), capped or fixed workspaces, shards, the
 // basic variant, or a split of the flat map that is not the default one.
 bool items_handle(const domagg_ctx* h) {
