@@ -398,8 +398,13 @@ __device__ __forceinline__ u32 cluster_size() {
     asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return r;
 }
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // The address of `p` (this block's shared memory) in block `rank` of the cluster.
 __device__ __forceinline__ u32 cluster_map(const void* p, u32 rank) {
@@ -417,6 +422,9 @@ __device__ __forceinline__ void cluster_st16(u32 a, unsigned short v) {
 template <int M, bool F32, int ITEMS, int T>
 __global__ __launch_bounds__(T) void k_pair_stats(const __grid_constant__ PairStatCall C) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // every block of the cluster has to have started before another stores
+    // into its shared memory: arrive here, wait behind the key loads
+    cluster_arrive();
     constexpr int W = T / 32, R = M - 1;
     constexpr u32 PER = T / RADIX;  // threads per digit, eight warps' counts each
     static_assert(PER * 8 == W && (PER == 1 || PER == 4), "digit scan");
@@ -462,6 +470,7 @@ __global__ __launch_bounds__(T) void k_pair_stats(const __grid_constant__ PairSt
         }
     }
     if (nan) atomicOr(&C.ctl->error, ERR_NAN);
+    cluster_wait();  // (the arrival at the kernel's start)
     u32 buf = 0;
 #pragma unroll 1
     for (int sh = 0; sh < 32; sh += 8) {
