@@ -88,6 +88,11 @@ struct domagg_ctx {
     int pre_bits = 32;
     void* h_pin = nullptr;
     size_t h_pin_cap = 0;
+    // copies out of h_pin that may still be queued when a call returns: a
+    // later call waits before it writes there (pin_acquire).  PIN_MARKED:
+    // ev_pin is behind the last of them; PIN_QUEUED: no event was recorded
+    enum PinState { PIN_IDLE, PIN_QUEUED, PIN_MARKED } pin_state = PIN_IDLE;
+    cudaEvent_t ev_pin = nullptr;
     std::string err;
     domagg_stats stats{};
     bool timing = false;
@@ -184,6 +189,7 @@ domagg_status grow_pinned(domagg_ctx* h, size_t bytes) {
     if (h->frozen) return fail(h, DOMAGG_ERR_OOM, "a planned run needs more pinned memory than its plan reserved");
     if (h->h_pin) {
         cudaDeviceSynchronize();
+        h->pin_state = domagg_ctx::PIN_IDLE;
         cudaFreeHost(h->h_pin);
         h->h_pin = nullptr;
     }
@@ -195,6 +201,23 @@ domagg_status grow_pinned(domagg_ctx* h, size_t bytes) {
     }
     h->h_pin_cap = want;
     return DOMAGG_OK;
+}
+
+// Before the host writes the pinned area: waits for the copies out of it that
+// an earlier call left queued (a call's record tables lie behind all of its
+// kernels up to the flat map, and the call has returned by then).
+void pin_acquire(domagg_ctx* h) {
+    if (h->pin_state == domagg_ctx::PIN_MARKED) cudaEventSynchronize(h->ev_pin);
+    else if (h->pin_state == domagg_ctx::PIN_QUEUED) cudaDeviceSynchronize();
+    h->pin_state = domagg_ctx::PIN_IDLE;
+}
+
+// Behind a call's last copy out of the pinned area.  (A fixed host area is
+// pageable: its copies have read it when they return.)
+void pin_mark(domagg_ctx* h, cudaStream_t s) {
+    if (h->no_alloc) return;
+    h->pin_state = h->ev_pin && cudaEventRecord(h->ev_pin, s) == cudaSuccess ? domagg_ctx::PIN_MARKED
+                                                                           : domagg_ctx::PIN_QUEUED;
 }
 
 // Checked build: the site of the first out-of-range index any kernel met
@@ -318,6 +341,7 @@ domagg_status run_wavelet(domagg_ctx* h, std::vector<Inst>& inst, Inst* d_inst, 
     L.stop();
     cudaError_t e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "point phase");
+    h->pin_state = domagg_ctx::PIN_IDLE;
     if (h_ctl->error) {
         const u32 bits = h_ctl->error;
         cudaMemsetAsync(&h->ctl->error, 0, sizeof(u32), stream);
@@ -804,6 +828,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         domagg_status st = grow_pinned(h, item_pos + (items ? 2 * sizeof(u32) * k * LMAX : 0) + 64);
         if (st) return st;
         hp = (char*)h->h_pin;
+        pin_acquire(h);
         memcpy(hp + lvl_bytes, inst.data(), sizeof(Inst) * k);
         u32* ho = (u32*)(hp + lvl_bytes + sizeof(Inst) * k);
         memcpy(ho, pt_offs.data(), sizeof(u32) * (k + 1));
@@ -814,6 +839,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             memcpy(ho + 4 * (k + 1), multi.data(), sizeof(u32) * multi.size());
         }
         cudaMemcpyAsync(d_inst, hp + lvl_bytes, up_bytes, cudaMemcpyHostToDevice, stream);
+        if (!h->no_alloc) h->pin_state = domagg_ctx::PIN_QUEUED;  // (until this call's synchronisation)
         maybe_reset_epochs(h, stream);
     }
 
@@ -970,6 +996,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             L.stop();
             e = cudaStreamSynchronize(stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "point phase");
+            h->pin_state = domagg_ctx::PIN_IDLE;
             if (const u32 site = bounds_site(true)) return bounds_error(h, site);
             h->ctl_host = *h_ctl;
             if (h_ctl->error) {
@@ -1086,6 +1113,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         L.stop();
         e = cudaStreamSynchronize(stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "point phase");
+        h->pin_state = domagg_ctx::PIN_IDLE;
         if (const u32 site = bounds_site(true)) return bounds_error(h, site);
         h->ctl_host = *h_ctl;
         if (h_ctl->error) {
@@ -1427,6 +1455,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         const bool records = planned || C.T > 0;
         if (records && !planned) {
             cudaMemcpyAsync(d_up, hb, sizeof(u32) * chunk_upload_words(C), cudaMemcpyHostToDevice, stream);
+            pin_mark(h, stream);
             maybe_reset_epochs(h, stream);
         }
         // fresh epoch and tile counters for the record phase of this chunk
@@ -1549,6 +1578,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         if (chunks.size() > 1 && !planned) {
             e = cudaStreamSynchronize(stream);  // the next chunk's host tables reuse the pinned area
             if (e != cudaSuccess) return cuda_fail(h, e, "record phase");
+            h->pin_state = domagg_ctx::PIN_IDLE;
         }
     }
     e = cudaGetLastError();
@@ -2053,6 +2083,10 @@ domagg_status domagg_create(domagg_handle* out, int device, size_t max_workspace
         delete h;
         return DOMAGG_ERR_CUDA;
     }
+    if (cudaEventCreateWithFlags(&h->ev_pin, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        h->ev_pin = nullptr;
+    }
     cudaMemset(h->ctl, 0, sizeof(Ctl));
     cudaDeviceSynchronize();
     *out = h;
@@ -2073,7 +2107,7 @@ domagg_status domagg_destroy(domagg_handle h) {
     for (cudaEvent_t e : h->pool) cudaEventDestroy(e);
     for (cudaStream_t s : h->aux)
         if (s) cudaStreamDestroy(s);
-    for (cudaEvent_t e : {h->ev_fork, h->ev_join[0], h->ev_join[1], h->ev_w})
+    for (cudaEvent_t e : {h->ev_fork, h->ev_join[0], h->ev_join[1], h->ev_w, h->ev_pin})
         if (e) cudaEventDestroy(e);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     delete h;
