@@ -23,7 +23,9 @@
  *     coordinate makes the call fail with DOMAGG_ERR_NAN.
  *   - Pointers marked "device" are CUDA device memory owned by the caller and
  *     must stay valid until the work on `stream` has finished.  The library
- *     never frees caller memory.
+ *     never frees caller memory.  An output may share memory with the inputs
+ *     (say out == d_weights): the inputs of a call, or of a batch's instances
+ *     of one m, are read before its outputs are written.
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream).  Device
  *     entry points enqueue work on it.  domagg_forward and domagg_backward
  *     synchronise the stream once in the call (they read the record count to

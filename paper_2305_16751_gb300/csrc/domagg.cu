@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <iterator>
 #include <mutex>
 #include <new>
 #include <string>
@@ -1658,6 +1659,39 @@ domagg_status run_m(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype 
 // ---------------------------------------------------------------------------
 // small problems by their definition (k_pairs.cuh)
 // ---------------------------------------------------------------------------
+size_t dtype_size(domagg_dtype t) { return t == DOMAGG_I64 ? 8 : 4; }
+
+size_t out_size(domagg_op op, domagg_dtype wt) {
+    if (op == DOMAGG_COUNT) return 8;
+    return dtype_size(wt);
+}
+
+// Whether an instance's output shares memory with any instance's input.  The
+// pipeline has read every input before it writes an output, so such calls are
+// right there; k_pairs writes a query tile while other blocks still read, and
+// a batch by pairs or in parts takes its instances in another order.
+// (Outputs do not overlap one another.)
+struct MemRange {
+    uintptr_t a, b;  // [a, b)
+    MemRange(const void* p, u64 bytes) : a((uintptr_t)p), b(a + bytes) {}
+};
+bool output_is_input(const std::vector<Inst>* groups, domagg_dtype wt, domagg_op op) {
+    std::vector<MemRange> outs;
+    const u64 ob = out_size(op, wt), wb = op == DOMAGG_COUNT ? 0 : dtype_size(wt);
+    for (int m = 1; m <= 4; ++m)
+        for (const Inst& I : groups[m]) outs.emplace_back(I.out, I.nQ * ob);
+    std::sort(outs.begin(), outs.end(), [](const MemRange& x, const MemRange& y) { return x.a < y.a; });
+    auto hit = [&](const MemRange& r) {
+        if (r.a == r.b) return false;
+        auto it = std::lower_bound(outs.begin(), outs.end(), r.b, [](const MemRange& x, uintptr_t v) { return x.a < v; });
+        return it != outs.begin() && std::prev(it)->b > r.a;
+    };
+    for (int m = 1; m <= 4; ++m)
+        for (const Inst& I : groups[m])
+            if (hit({I.dw, I.nD * wb}) || hit({I.dco, (u64)I.nD * m * 4}) || hit({I.qco, (u64)I.nQ * m * 4})) return true;
+    return false;
+}
+
 // Where the line lies: a problem of at most PSTAT_MAX points (its statistics
 // then fit one cluster's shared memory), that is at most 1.5e8 pairs
 // (|D| x |Q|): 63e6 pairs of m = 3 take 30 us, where the pipeline's launches
@@ -1908,9 +1942,13 @@ domagg_status run_pairs_one(domagg_ctx* h, int m, const Inst& I, domagg_dtype ct
 domagg_status dispatch(domagg_ctx* h, int m, std::vector<Inst>& inst, domagg_dtype ct, domagg_dtype wt,
                        domagg_op op, bool negate, cudaStream_t s, const Planned* pl, bool pairs, bool items) {
     if (pairs && !pl && inst.size() == 1 && pairs_allowed(h, m, inst[0]) && pairs_fit(inst[0])) {
-        const domagg_status st = run_pairs_one(h, m, inst[0], ct, wt, op, negate, s);
-        if (st != DOMAGG_ERR_OOM) return st;
-        h->err.clear();  // the pipeline may fit a capped workspace that the pairs' partials do not
+        std::vector<Inst> one[5];
+        one[m] = inst;
+        if (!output_is_input(one, wt, op)) {
+            const domagg_status st = run_pairs_one(h, m, inst[0], ct, wt, op, negate, s);
+            if (st != DOMAGG_ERR_OOM) return st;
+            h->err.clear();  // the pipeline may fit a capped workspace that the pairs' partials do not
+        }
     }
     if (op == DOMAGG_COUNT) return run_m<OpCount>(h, m, inst, ct, negate, s, pl, items);
     if (op == DOMAGG_SUM && wt == DOMAGG_F32) return run_m<OpSumF32>(h, m, inst, ct, negate, s, pl, items);
@@ -1971,13 +2009,6 @@ domagg_status check_common(domagg_ctx* h, int m, int64_t nD, int64_t nQ, domagg_
     if ((op == DOMAGG_MAX || op == DOMAGG_MIN) && wt != DOMAGG_I32 && wt != DOMAGG_F32)
         return fail(h, DOMAGG_ERR_INVALID_ARG, "MAX takes i32 or f32 weights");
     return DOMAGG_OK;
-}
-
-size_t dtype_size(domagg_dtype t) { return t == DOMAGG_I64 ? 8 : 4; }
-
-size_t out_size(domagg_op op, domagg_dtype wt) {
-    if (op == DOMAGG_COUNT) return 8;
-    return dtype_size(wt);
 }
 
 Inst make_inst(const void* dco, int64_t nD, const void* qco, int64_t nQ, const void* dw, void* out) {
@@ -2356,7 +2387,8 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst, 
     cudaSetDevice(h->device);
     // the small instances by pairs (enqueued first, synchronised with the others)
     std::vector<Inst> small[5];
-    {
+    const bool in_place = output_is_input(groups, weight_dtype, op);
+    if (!in_place) {
         std::vector<Inst> all[5];
         for (int m = 1; m <= 4; ++m) all[m] = groups[m];
         if (pairs_split(h, groups, small)) {
@@ -2379,7 +2411,8 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst, 
         if (groups[m].empty()) continue;
         // one call per group of at most 2^31 - 1 points (m = 3: as many as may
         // go by items; the statistics are the group's)
-        const int64_t most = m == 3 && items_handle(h) ? (int64_t)ITEM_MAX_POINTS : ((int64_t)1 << 31) - 1;
+        const int64_t most =
+            m == 3 && items_handle(h) && !in_place ? (int64_t)ITEM_MAX_POINTS : ((int64_t)1 << 31) - 1;
         std::vector<Inst> part;
         domagg_stats sum;
         memset(&sum, 0, sizeof(sum));
@@ -2669,7 +2702,8 @@ domagg_status domagg_batch_plan(domagg_plan* out, int device, int k, const domag
         delete p;
         return DOMAGG_ERR_INVALID_ARG;
     }
-    if (const domagg_status st = plan_pairs(p, groups, (cudaStream_t)stream)) {
+    const bool in_place = output_is_input(groups, weight_dtype, op);
+    if (const domagg_status st = in_place ? DOMAGG_OK : plan_pairs(p, groups, (cudaStream_t)stream)) {
         g_plan_create_error = p->err;
         plan_free(p);
         return st;
