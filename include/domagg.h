@@ -139,11 +139,12 @@ domagg_status domagg_forward_ex(domagg_handle h, int m, const void* d_coords, in
  * paper's Sec. 6 reading: the flat map is partitioned and one exchange of the
  * outputs joins the parts).  Every shard runs the point phase on all points
  * (ranks, the order of the last coordinate); the flat map's records are
- * split by node: with gS the rank levels taken per group of 2^gS ranks in
- * shared memory (m = 2; 0 otherwise), shard s takes the levels lv >= gS of
+ * split by node: with gS the rank levels taken per group of 2^gS ranks
+ * (m = 2, 3; 0 otherwise), shard s takes the levels lv >= gS of
  * the first rank with (lv - gS) % nshards == s and the groups g with
  * g % nshards == s (m = 1 has a single level: shard 0 takes it and the
- * others return the unit).  The shard's outputs are F over its records only;
+ * others return the unit).  gS depends on the data and the handle's knobs
+ * only, so the shards may run on handles of different workspace caps.  The shard's outputs are F over its records only;
  * F over the nshards outputs (domagg_combine, or a collective with F) is
  * domagg_forward's result.
  *   shard, nshards  0 <= shard < nshards <= 64

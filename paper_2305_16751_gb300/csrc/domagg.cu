@@ -1016,8 +1016,10 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     }
     // ---- the levels whose records go through HBM (this shard's, and for
     // m = 2 the levels above the groups of ranks that k_group takes)
-    // points of a group on average, at most (one group per SM for few points)
-    const bool tight = h->no_alloc || h->max_ws > 0;
+    // points of a group on average, at most (one group per SM for few points).
+    // Shards have to agree on the groups whatever handle and device they run
+    // on: no limit that depends on either
+    const bool tight = h->no_alloc || h->max_ws > 0 || inst[0].nshards > 0;
     const u32 gavg = M == 3 ? g3_avg(N, tight, items) : group_avg(N, h->sms, h->top_bits == TOP_MAX_BITS && !tight);
     L.start(KIND_SMALL, 0.0);
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,

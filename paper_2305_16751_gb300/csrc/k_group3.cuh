@@ -39,8 +39,8 @@ constexpr u32 G3_CAP = 10240;
 // 4096 ranks, fewer where there are few points, so that the query tiles still
 // cover the chip (1e5 per side: 677 us with N / 64, 773 with N / 512).  No
 // limit of its own (8192 ranks, a level of records less) where room for
-// records is short: a workspace that is capped or fixed, and calls that come
-// near the limit of 2^32 records.
+// records is short (a workspace that is capped or fixed, and calls that come
+// near the limit of 2^32 records) and for a shard.
 __host__ __device__ constexpr u32 g3_avg(u64 N, bool tight, bool items) {
     const u64 c = N / 64u;
     if (tight || (!items && N > (1ull << 24))) return 0xffffffffu;
