@@ -145,6 +145,25 @@ domagg_status cuda_fail(domagg_ctx* h, cudaError_t e, const char* where) {
     return fail(h, DOMAGG_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
+void free_buffer(DevBuf& b) {
+    if (b.p) cudaFree(b.p);
+    b = DevBuf{};
+}
+
+// Gives back what the handle holds for another route than the one that needs
+// buffer b: the small problems' buffers (their kernels, if any, end first).
+// Returns whether anything was freed.
+bool release_idle(domagg_ctx* h, const DevBuf& b) {
+    bool any = false;
+    if (&b != &h->pairs && &b != &h->st_pairs && (h->pairs.p || h->st_pairs.p)) {
+        cudaDeviceSynchronize();
+        free_buffer(h->pairs);
+        free_buffer(h->st_pairs);
+        any = true;
+    }
+    return any;
+}
+
 // Grows a device buffer to at least `bytes` (contents are not kept).  Status
 // buffers are zeroed when (re)allocated: fresh memory may hold old data of
 // this process, and a stale word must never look like a status of the
@@ -156,6 +175,7 @@ domagg_status grow(domagg_ctx* h, DevBuf& b, size_t bytes, bool zero = false) {
     size_t want = std::max(bytes, b.cap + b.cap / 4);
     if (h->max_ws && h->held() - b.cap + want > h->max_ws) {
         want = bytes;
+        if (h->held() - b.cap + want > h->max_ws) release_idle(h, b);
         if (h->held() - b.cap + want > h->max_ws)
             return fail(h, DOMAGG_ERR_OOM, "workspace would exceed max_workspace_bytes");
     }
@@ -1166,7 +1186,9 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                 const double per_rec = 2.0 * sizeof(K) + 2.0 * sizeof(Pay) + sizeof(Part) + 8.0;
                 double budget = std::max(0.6 * (double)free_b + (double)h->recs.cap, 2.0e9);
                 // a capped handle also caps the records of one chunk
-                if (h->max_ws) budget = std::min(budget, 0.5 * (double)(h->max_ws - std::min(h->max_ws, h->held() - h->recs.cap)));
+                // (the small problems' buffers are given back if need be)
+                const size_t others = h->held() - h->recs.cap - h->pairs.cap - h->st_pairs.cap;
+                if (h->max_ws) budget = std::min(budget, 0.5 * (double)(h->max_ws - std::min(h->max_ws, others)));
                 chunk_cap = std::max<u64>(1, std::min<u64>(chunk_cap, (u64)(budget / per_rec)));
             } else {
                 cudaGetLastError();
