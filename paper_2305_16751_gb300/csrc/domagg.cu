@@ -81,6 +81,7 @@ struct domagg_ctx {
     // m = 3: the levels above the groups as m = 2 problems (k_items.cuh), on a
     // handle of their own; tuning knob "nodes" (1: by size, 2: always)
     DevBuf items;
+    bool items_live = false;  // between the nodes' stage and the end of its call
     domagg_ctx* sub = nullptr;
     int nodes = 1;
     // on that handle: the point phase's input, ready-made (ranked keys of at
@@ -150,11 +151,27 @@ void free_buffer(DevBuf& b) {
     b = DevBuf{};
 }
 
+void free_buffers(domagg_ctx* h) {
+    for (DevBuf* b : {&h->pts, &h->recs, &h->st_multi, &h->st_seg, &h->stage, &h->st_wv, &h->pairs, &h->st_pairs,
+                      &h->items})
+        free_buffer(*b);
+}
+
+// Gives back what the nodes of m = 3 hold: their items and their handle's
+// buffers (the handle itself stays).
+bool release_nodes(domagg_ctx* h) {
+    if (!h->items.p && !(h->sub && h->sub->held())) return false;
+    cudaDeviceSynchronize();
+    free_buffer(h->items);
+    if (h->sub) free_buffers(h->sub);
+    return true;
+}
+
 // Gives back what the handle holds for another route than the one that needs
-// buffer b: the small problems' buffers (their kernels, if any, end first).
-// Returns whether anything was freed.
+// buffer b: the small problems' buffers (their kernels, if any, end first),
+// and the nodes' unless they are in use.  Returns whether anything was freed.
 bool release_idle(domagg_ctx* h, const DevBuf& b) {
-    bool any = false;
+    bool any = !h->items_live && &b != &h->items && release_nodes(h);
     if (&b != &h->pairs && &b != &h->st_pairs && (h->pairs.p || h->st_pairs.p)) {
         cudaDeviceSynchronize();
         free_buffer(h->pairs);
@@ -188,6 +205,10 @@ domagg_status grow(domagg_ctx* h, DevBuf& b, size_t bytes, bool zero = false) {
     if (e != cudaSuccess) {
         cudaGetLastError();
         e = cudaMalloc(&b.p, bytes);
+        if (e != cudaSuccess && release_idle(h, b)) {
+            cudaGetLastError();
+            e = cudaMalloc(&b.p, bytes);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             b.p = nullptr;
@@ -554,6 +575,7 @@ domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& ins
     };
     Carver c0(nullptr);
     carve(c0);
+    h->items_live = true;
     domagg_status st = grow(h, h->items, c0.off);
     if (!st) st = grow(h, h->st_multi, (size_t)tiles_of(sizes, SORT_MIN_TILE) * RADIX * sizeof(u64), true);
     if (!st) st = grow_pinned_tables(h, sizeof(u32) * (up_words + 2 * nodes + 1));
@@ -1659,11 +1681,13 @@ domagg_status run_ct(domagg_ctx* h, std::vector<Inst>& inst, domagg_dtype ct, bo
             std::vector<Inst> I = inst;
             const domagg_status st = ct == DOMAGG_F32 ? run<M, Op, true>(h, I, negate, s, nullptr, true)
                                                       : run<M, Op, false>(h, I, negate, s, nullptr, true);
+            h->items_live = false;
             if (st != DOMAGG_ERR_OOM) {
                 inst.swap(I);
                 return st;
             }
-            h->err.clear();  // too many nodes, or no room for the items: the records
+            h->err.clear();  // too many nodes, or no room for the items: the records, in the room the nodes held
+            release_nodes(h);
         }
     }
     return ct == DOMAGG_F32 ? run<M, Op, true>(h, inst, negate, s, pl) : run<M, Op, false>(h, inst, negate, s, pl);
@@ -2152,9 +2176,7 @@ domagg_status domagg_destroy(domagg_handle h) {
     if (!h) return DOMAGG_ERR_INVALID_ARG;
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
-    for (DevBuf* b : {&h->pts, &h->recs, &h->st_multi, &h->st_seg, &h->stage, &h->st_wv, &h->pairs, &h->st_pairs,
-                      &h->items})
-        if (b->p) cudaFree(b->p);
+    free_buffers(h);
     if (h->sub) domagg_destroy(h->sub);
     if (h->ctl) cudaFree(h->ctl);
     if (h->h_pair) cudaFreeHost(h->h_pair);
