@@ -511,7 +511,9 @@ struct ItemStage {
     u32 n_part = 0;
     const u32* qseg = nullptr;
 };
-// DOMAGG_ERR_OOM: too many nodes or no room; the caller takes the records.
+// (An instance with more nodes than its share of ITEM_MAX_NODES is left to the
+// records by k_group_plan.)  DOMAGG_ERR_OOM: no room; the caller takes the
+// records.
 template <class Op>
 domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& inst, ItemStage& S) {
     typedef typename Op::W W;
@@ -1067,7 +1069,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,
                                             govf, M == 3 ? G3_CAP : group_cap(gavg), gavg,
                                             use_groups ? h->group_bits : 0,
-                                            use_top ? h->top_bits : 0, items ? 1 : 0, rec_all,
+                                            use_top ? h->top_bits : 0, items ? (ITEM_MAX_NODES << 32) / N : 0, rec_all,
                                             use_groups && k == 1 ? gslot : nullptr);
     L.stop();
     // ---- count / offset scan of the flat map, per level
@@ -1686,7 +1688,7 @@ domagg_status run_ct(domagg_ctx* h, std::vector<Inst>& inst, domagg_dtype ct, bo
                 inst.swap(I);
                 return st;
             }
-            h->err.clear();  // too many nodes, or no room for the items: the records, in the room the nodes held
+            h->err.clear();  // no room for the items: the records, in the room the nodes held
             release_nodes(h);
         }
     }

@@ -86,7 +86,8 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // [gS, tS) through the records in HBM (lvmask); both masks hold this
 // shard's levels only.
 // rstart (per instance, at pt_off + s) holds the rank-sorted position of the
-// first point of every (undoubled) rank, and n at index U.  A non-strict
+// first point of every (undoubled) rank, and n at index U.  node_share: nodes
+// per point the call's nodes' path takes (m = 3, in 2^-32; 0: none).  A non-strict
 // first coordinate doubles the ranks (2r for data, 2r+1 for queries), so a
 // group of 2^gS ranks is 2^(gS-1) undoubled ranks.  Also writes gbits[s],
 // the bits the group sort sorts: the group id's (b0 - gS) and, for m = 3, the
@@ -94,7 +95,7 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
-                                                    u32 cap, u32 avg, int max_bits, int top_bits, int items,
+                                                    u32 cap, u32 avg, int max_bits, int top_bits, u64 node_share,
                                                     unsigned long long* __restrict__ rec_all,
                                                     u32* __restrict__ gslot_off) {
     __shared__ u32 s_ovf[32];
@@ -165,7 +166,13 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
                 if (lv >= tS) tmask |= 1u << lv;
                 else mask |= 1u << lv;
             }
-        if (M == 3 && items) {  // the levels above the groups by items (k_items.cuh)
+        // the levels above the groups by items (k_items.cuh), if their nodes
+        // (2^(b0 - gS) - 1 at most) lie within the instance's share of the
+        // limit; decided here, before the records are counted, since a call
+        // found to hold too many afterwards would start again (a third of the
+        // points on one value, so without groups, and the others spread: as
+        // many nodes as ranks)
+        if (M == 3 && mask && (1ull << (b0 - chosen)) - 1ull <= (((u64)n * node_share) >> 32)) {
             tmask = mask;
             mask = 0;
         }
