@@ -518,9 +518,10 @@ template <class Op>
 domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& inst, ItemStage& S) {
     typedef typename Op::W W;
     typedef typename Op::Out Out;
-    typedef typename Op::Part Part;
+    typedef typename Op::Acc Acc;
     constexpr int WT = OpTraits<Op>::WT;
     constexpr size_t WB = WT == 3 ? 0 : sizeof(W);
+    constexpr bool FF = std::is_same<Op, OpSumF32>::value;
     const cudaStream_t stream = L.stream;
     const int k = S.k;
     // segments: the levels of every instance, with items
@@ -573,7 +574,8 @@ domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& ins
         R[16] = c.take<u32>(T);
         R[17] = c.take<char>((size_t)(T - Q) * WB);
         R[18] = c.take<Out>(Q);
-        R[19] = c.take<Part>(Q);
+        R[19] = c.take<Acc>(Q);
+        R[20] = c.take<float>(FF ? Q : 0);  // the low halves of float32 sums
     };
     Carver c0(nullptr);
     carve(c0);
@@ -657,6 +659,7 @@ domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& ins
         memset(&I, 0, sizeof(I));
         I.dw = WT == 3 ? nullptr : (const char*)R[17] + da * WB;
         I.out = (Out*)R[18] + qa;
+        I.out_lo = FF ? (float*)R[20] + qa : nullptr;  // a float-float pair, as a shard's
         I.nD = (u32)nD;
         I.nQ = (u32)nQ;
         sub.push_back(I);
@@ -673,8 +676,9 @@ domagg_status run_items(domagg_ctx* h, Launcher& L, const std::vector<Inst>& ins
         if (st) return fail(h, st, "nodes: " + h->sub->err);
     }
     if (Q > 0) {
-        L.start(KIND_REDUCE, (double)Q * (sizeof(Out) + 4 + sizeof(Part)));
-        k_item_out<Op><<<qgrid, 256, 0, stream>>>((const Out*)R[18], (const u32*)R[15], (u32)Q, (Part*)R[19]);
+        L.start(KIND_REDUCE, (double)Q * (sizeof(Out) + (FF ? 4 : 0) + 4 + sizeof(Acc)));
+        k_item_out<Op><<<qgrid, 256, 0, stream>>>((const Out*)R[18], (const float*)R[20], (const u32*)R[15], (u32)Q,
+                                                  (Acc*)R[19]);
         L.stop();
     }
     S.part = R[19];
@@ -1616,7 +1620,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             L.start(KIND_REDUCE, (double)C.Tq * sizeof(Part) + (double)(qe - qb) * (8 + sizeof(typename Op::Out)));
             k_reduce<Op, M><<<grid, 256, 0, stream>>>(d_chunk_off, k, C.k0, C.k1, d_pt_offs, pr0, pr1, pr2, pj,
                                                       qchunk_base, d_pt_tiles, (const u32*)P[25], d_qsbase, d_inst,
-                                                      partial, (u32)C.Tq, gacc, govf, (const Part*)IS.part, IS.n_part,
+                                                      partial, (u32)C.Tq, gacc, govf, (const typename Op::Acc*)IS.part, IS.n_part,
                                                       (const u32*)P[60], (const u32*)P[61],
                                                       IS.qseg ? IS.qseg + (size_t)C.k0 * LMAX : nullptr);
             L.stop();

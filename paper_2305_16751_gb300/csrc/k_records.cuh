@@ -725,7 +725,7 @@ __global__ __launch_bounds__(256) void k_reduce(const u32* __restrict__ chunk_of
                                                 const typename Op::Part* __restrict__ partial, u32 n_partial,
                                                 const typename Op::Part* __restrict__ gacc,
                                                 const unsigned char* __restrict__ govf,
-                                                const typename Op::Part* __restrict__ ipart, u32 n_ipart,
+                                                const typename Op::Acc* __restrict__ ipart, u32 n_ipart,
                                                 const u32* __restrict__ iqchunk_base,
                                                 const u32* __restrict__ itile_excl,
                                                 const u32* __restrict__ iqseg_base /*[k1-k0][LMAX]*/) {
@@ -809,8 +809,8 @@ __global__ __launch_bounds__(256) void k_reduce(const u32* __restrict__ chunk_of
             }
         }
         if (M == 3 && ipart) {
-            // the levels taken by items: one partial per query and level, in
-            // slots as for m = 2
+            // the levels taken by items: one answer per query and level (float
+            // sums: a float-float pair), in slots as for m = 2
             const u32 ibits = q ? pr0[p] & low_mask(I.b[0]) & I.topmask : 0u;
             __syncwarp();
             s_base[warp][lane] = __ldg(iqseg_base + (u64)(s - k0) * LMAX + lane) +
@@ -825,7 +825,7 @@ __global__ __launch_bounds__(256) void k_reduce(const u32* __restrict__ chunk_of
                 const u32 lv = __ffs(rem) - 1;
                 rem &= rem - 1;
                 const u32 slot = s_base[warp][lv] + (u32)__popc(s_mask[warp][lv] & lt);
-                if (domagg_check(slot < n_ipart, SITE_REDUCE)) acc = Op::F(acc, Op::from_part(ipart[slot]));
+                if (domagg_check(slot < n_ipart, SITE_REDUCE)) acc = Op::F(acc, ipart[slot]);
             }
         }
         if (q) {
