@@ -303,7 +303,7 @@ const char* domagg_last_error(domagg_handle h);
 typedef struct {
     int64_t n_points;      /* nD + nQ */
     int64_t n_records;     /* T: records of the flat map */
-    int64_t n_query_records; /* records that came from queries */
+    int64_t n_query_records; /* records that came from queries (m = 2, 3: those that went through HBM) */
     int32_t m;
     int32_t rank_bits[3];  /* b_i = ceil(log2 U_i) for the first m-1 dimensions */
     int64_t distinct[3];   /* U_i */

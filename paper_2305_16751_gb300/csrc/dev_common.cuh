@@ -37,6 +37,7 @@ struct Ctl {
     // (k_pair_stats): records so far (never reset) and, of the last single
     // problem, the distinct values and rank digits per coordinate
     unsigned long long pair_T[4];
+    unsigned long long pair_Tq;  // m = 4: of those, the queries'
     u32 pair_U[4][3], pair_b[4][3];
 };
 

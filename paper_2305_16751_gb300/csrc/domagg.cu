@@ -76,7 +76,7 @@ struct domagg_ctx {
     void* h_pair = nullptr;  // pinned: the tables, then the control block read back
     size_t h_pair_cap = 0;
     Ctl ctl_host{};            // the control block as last read back
-    u64 pair_T_seen[4] = {0, 0, 0, 0};  // Ctl::pair_T already accounted for
+    u64 pair_T_seen[4] = {0, 0, 0, 0}, pair_Tq_seen = 0;  // Ctl::pair_T, pair_Tq already accounted for
     bool use_pairs = true;     // tuning knob "pairs"
     // m = 3: the levels above the groups as m = 2 problems (k_items.cuh), on a
     // handle of their own; tuning knob "nodes" (1: by size, 2: always)
@@ -1954,11 +1954,16 @@ void pairs_stats(domagg_ctx* h, int m, const std::vector<Inst>& small, bool add)
     const Ctl& c = h->ctl_host;
     domagg_stats& S = h->stats;
     if (!add) memset(&S, 0, sizeof(S));
-    u64 n = 0;
-    for (const Inst& I : small) n += (u64)I.nD + I.nQ;
+    u64 n = 0, nQ = 0;
+    for (const Inst& I : small) {
+        n += (u64)I.nD + I.nQ;
+        nQ += I.nQ;
+    }
     const u64 T = m == 1 ? n : c.pair_T[m - 1] - h->pair_T_seen[m - 1];
+    const u64 Tq = m == 1 ? nQ : (m == 4 ? c.pair_Tq - h->pair_Tq_seen : 0);
     S.n_points += (int64_t)n;
     S.n_records += (int64_t)T;
+    S.n_query_records += (int64_t)Tq;
     S.n_records_shared += (int64_t)T;
     S.m = m;
     if (add) return;
@@ -1978,6 +1983,7 @@ void pairs_stats(domagg_ctx* h, int m, const std::vector<Inst>& small, bool add)
 
 void pairs_seen(domagg_ctx* h) {
     for (int i = 0; i < 4; ++i) h->pair_T_seen[i] = h->ctl_host.pair_T[i];
+    h->pair_Tq_seen = h->ctl_host.pair_Tq;
 }
 
 // A single small problem: the pairs, one synchronisation, the statistics.

@@ -592,7 +592,7 @@ __global__ __launch_bounds__(T) void k_pair_stats(const __grid_constant__ PairSt
     }
     const u32 U = (all + 1u) << ns;  // (a non-strict coordinate: 2r for data, 2r + 1 for queries)
     const u32 bits = U <= 1u ? 0u : 32u - __clz(U - 1u), mask = low_mask(bits);
-    unsigned long long sum = 0;
+    unsigned long long sum = 0, sum_q = 0;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
         const u32 p = p0 + 32u * j;
@@ -623,6 +623,7 @@ __global__ __launch_bounds__(T) void k_pair_stats(const __grid_constant__ PairSt
 #pragma unroll
             for (int e = 0; e < R; ++e) c *= (u32)__ldcg(C.cnt + o0 + C.total * (u64)e + i);
             sum += c;
+            if (R == 3 && i < nQ) sum_q += c;
         }
     }
     for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -632,6 +633,10 @@ __global__ __launch_bounds__(T) void k_pair_stats(const __grid_constant__ PairSt
         unsigned long long t = 0;
         for (int w = 0; w < W; ++w) t += s_sum[w];
         if (t) atomicAdd(&C.ctl->pair_T[M - 1], t);  // (never reset: the host takes differences)
+    }
+    if constexpr (R == 3) {
+        for (int o = 16; o >= 1; o >>= 1) sum_q += __shfl_xor_sync(0xffffffffu, sum_q, o);
+        if (lane == 0 && sum_q) atomicAdd(&C.ctl->pair_Tq, sum_q);
     }
 }
 
