@@ -389,8 +389,9 @@ domagg_status domagg_forward_noalloc(int m, const void* d_coords, int64_t nD, co
  *                    their defaults; 0 sends them through the pipeline;
  *   "nodes"          0, 1 or 2 (default 1): for m = 3, the first rank's levels
  *                    above the groups as one m = 2 problem per node, instead
- *                    of records in HBM; 1: calls of 2^19 to 2^25 points, 2:
- *                    up to 2^25 (never with a capped workspace, in a plan or a
+ *                    of records in HBM; 1: calls of 2^19 to 2^25 points,
+ *                    where the coordinates have distinct values enough to
+ *                    gain, 2: up to 2^25 (never with a capped workspace, in a plan or a
  *                    shard, or with group_bits off its default).  These calls
  *                    synchronise the stream twice more;
  *   "rank_windows"   0 .. 64 (default 0: about 48 MB of ranks each): windows

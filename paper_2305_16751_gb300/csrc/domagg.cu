@@ -500,6 +500,15 @@ domagg_status grow_pinned_tables(domagg_ctx* h, size_t bytes) {
 // a partial per (level, query item), at qseg[instance][level] + the query's
 // place in the level.
 constexpr u64 ITEM_MAX_NODES = 1u << 17, ITEM_MIN_POINTS = 1u << 19, ITEM_MAX_POINTS = 1u << 25;
+// Points x levels above the groups x (bits of the second rank - 6) from which
+// on the nodes gain.  Measured over 2^19 to 2^22 points, 1 to 12 levels and 1
+// to 22 bits, spread and tied: nodes against records 0.86 at 4.8e7 (5.2e5
+// points, 7 levels, 19 bits), 1.07 at 2.2e7 (12 bits), 1.27 at 4.19e7 (1e6
+// points, ties in both coordinates, 10 levels, 10 bits), 1.31 at 3.2e7 (the
+// same at 8e5), 0.96 at 5.7e7 (2e6 points, 9 levels, 9 bits), 1.00 at 8.4e7
+// (2e6 points, the ties again), 1.01 at 1.9e7 (7 bits), 1.4 with two values in
+// the first coordinates
+constexpr u64 ITEM_MIN_GAIN = 42000000;
 struct ItemStage {
     int k;
     const std::vector<u32>*lvl, *qlvl;  // items and query items per (instance, level)
@@ -1073,7 +1082,8 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     k_group_plan<M><<<k, 1024, 0, stream>>>(d_inst, use_groups ? rstart : nullptr, use_groups ? gbits : nullptr,
                                             govf, M == 3 ? G3_CAP : group_cap(gavg), gavg,
                                             use_groups ? h->group_bits : 0,
-                                            use_top ? h->top_bits : 0, items ? (ITEM_MAX_NODES << 32) / N : 0, rec_all,
+                                            use_top ? h->top_bits : 0, items ? (ITEM_MAX_NODES << 32) / N : 0,
+                                            h->nodes == 2 ? 0u : (u32)((ITEM_MIN_GAIN + N - 1) / N), rec_all,
                                             use_groups && k == 1 ? gslot : nullptr);
     L.stop();
     // ---- count / offset scan of the flat map, per level

@@ -87,15 +87,17 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // shard's levels only.
 // rstart (per instance, at pt_off + s) holds the rank-sorted position of the
 // first point of every (undoubled) rank, and n at index U.  node_share: nodes
-// per point the call's nodes' path takes (m = 3, in 2^-32; 0: none).  A non-strict
+// per point the call's nodes' path takes (m = 3, in 2^-32; 0: none); node_min:
+// ITEM_MIN_GAIN over the call's points (0: no such limit).  A non-strict
 // first coordinate doubles the ranks (2r for data, 2r+1 for queries), so a
 // group of 2^gS ranks is 2^(gS-1) undoubled ranks.  Also writes gbits[s],
 // the bits the group sort sorts: the group id's (b0 - gS) and, for m = 3, the
 // role's.
+constexpr u32 ITEM_FREE_BITS = 6;  // bits of the second rank whose records cost what an item costs
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
-                                                    u32 cap, u32 avg, int max_bits, int top_bits, u64 node_share,
+                                                    u32 cap, u32 avg, int max_bits, int top_bits, u64 node_share, u32 node_min,
                                                     unsigned long long* __restrict__ rec_all,
                                                     u32* __restrict__ gslot_off) {
     __shared__ u32 s_ovf[32];
@@ -171,8 +173,12 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
         // limit; decided here, before the records are counted, since a call
         // found to hold too many afterwards would start again (a third of the
         // points on one value, so without groups, and the others spread: as
-        // many nodes as ranks)
-        if (M == 3 && mask && (1ull << (b0 - chosen)) - 1ull <= (((u64)n * node_share) >> 32)) {
+        // many nodes as ranks).  And if the records they replace, a level's
+        // item for half of the second rank's bits each, are enough to pay for
+        // the items and the nodes' launches (ITEM_MIN_GAIN)
+        const u32 b1 = I.b[1];
+        if (M == 3 && mask && (1ull << (b0 - chosen)) - 1ull <= (((u64)n * node_share) >> 32) &&
+            (node_min == 0u || (b1 > ITEM_FREE_BITS && (b0 - chosen) * (b1 - ITEM_FREE_BITS) >= node_min))) {
             tmask = mask;
             mask = 0;
         }
