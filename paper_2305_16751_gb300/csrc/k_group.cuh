@@ -75,7 +75,8 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // Per instance (one block each): the largest gS <= min(GROUP_MAX_BITS, b0)
 // whose groups of 2^gS ranks that hold more than `cap` points each (too
 // many for shared memory: heavy ties) hold at most a quarter of the points
-// and which hold at most `avg` points on average, and the number of groups G (m = 2: k_group; m = 3: k_group3); gS = 0 (no
+// and which hold at most `avg` points on average (m = 3 with such a limit: and
+// whose pairs pay, G3_PAIRS_PER_BIT), and the number of groups G (m = 2: k_group; m = 3: k_group3); gS = 0 (no
 // level in groups) if no width qualifies, or if the instance takes another
 // path.  m = 2 prefers the widest without any group above `cap`, where the
 // levels from there up still fit the top tiles: overflowing groups' records
@@ -93,6 +94,14 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // group of 2^gS ranks is 2^(gS-1) undoubled ranks.  Also writes gbits[s],
 // the bits the group sort sorts: the group id's (b0 - gS) and, for m = 3, the
 // role's.
+// m = 3: a point of a group of c points meets c / 8 pairs, 6e-8 c us at 2.1e6
+// pairs per us, and spares a level's records, b1 / 4 of them at 4e-5 us, for
+// each of the S levels below the group: a width pays while c (over the points)
+// is at most 160 S b1.  (6e5 points, 200 first ranks, S = 1 and 6000 points a
+// group: 748 us without groups, 969 with, second ranks of 8 bits; 1072 and
+// 1230 of 20 bits.  1.9e6 points in 24 instances of 200 ranks, S = 4, 6400
+// points: 2473 us, 2691 at S = 2, of 20 bits; 1856 and 1764 of 5 bits.)
+constexpr u32 G3_PAIRS_PER_BIT = 160;
 constexpr u32 ITEM_FREE_BITS = 6;  // bits of the second rank whose records cost what an item costs
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
@@ -101,6 +110,7 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
                                                     unsigned long long* __restrict__ rec_all,
                                                     u32* __restrict__ gslot_off) {
     __shared__ u32 s_ovf[32];
+    __shared__ u64 s_sq[32];
     const int s = blockIdx.x;
     Inst& I = inst[s];
     const u32 n = I.nD + I.nQ;
@@ -115,18 +125,31 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
         const u32 us = (u32)S - ns;  // undoubled ranks per group: 2^us
         const u32 g_n = (Uu + (1u << us) - 1u) >> us;
         u32 ov = 0;  // points in groups too large for shared memory
+        u64 sq = 0;  // m = 3: the other groups' points, squared
         for (u32 g = threadIdx.x; g < g_n; g += blockDim.x) {
             const u32 lo = g << us, hi = min((g + 1u) << us, Uu);
             const u32 c = __ldg(rs + hi) - __ldg(rs + lo);
             if (c > cap) ov += c;
+            else if (M == 3) sq += (u64)c * c;
         }
-        for (int o = 16; o >= 1; o >>= 1) ov += __shfl_xor_sync(0xffffffffu, ov, o);
+        for (int o = 16; o >= 1; o >>= 1) {
+            ov += __shfl_xor_sync(0xffffffffu, ov, o);
+            if (M == 3) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        }
         __syncthreads();
-        if ((threadIdx.x & 31) == 0) s_ovf[threadIdx.x >> 5] = ov;
+        if ((threadIdx.x & 31) == 0) {
+            s_ovf[threadIdx.x >> 5] = ov;
+            s_sq[threadIdx.x >> 5] = sq;
+        }
         __syncthreads();
         ov = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) ov += s_ovf[w];
-        const bool ok = ov <= n / 4u && n <= (u64)avg * g_n;
+        sq = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            ov += s_ovf[w];
+            sq += s_sq[w];
+        }
+        bool ok = ov <= n / 4u && n <= (u64)avg * g_n;
+        if (M == 3 && avg != 0xffffffffu) ok = ok && sq <= (u64)n * (G3_PAIRS_PER_BIT * (u32)S * I.b[1]);
         if (ok && (!chosen || ov == 0u)) chosen = (u32)S;
         // m = 2: on to a narrower width without overflow, as long as the
         // levels above it fit the top tiles
