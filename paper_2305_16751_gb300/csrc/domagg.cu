@@ -48,7 +48,7 @@ struct Carver {
     T* take(size_t n) {
         off = (off + 255) & ~(size_t)255;
         T* r = base ? reinterpret_cast<T*>(base + off) : nullptr;
-        off += n * sizeof(T) + 64;  // slack: 16-byte-aligned bulk reads may run past the end
+        off += n * sizeof(T) + 64;  // (pieces do not touch)
         return r;
     }
 };
@@ -770,7 +770,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     // record counts (per level, of queries, per instance) and the instance
     // table, read back in one copy; the table and the offsets, uploaded in one
     const size_t lvl_bytes = 2 * sizeof(u32) * k * LMAX + sizeof(unsigned long long) * k;
-    const size_t off_bytes = 3 * sizeof(u32) * (k + 1) + (use_top ? sizeof(u32) * (2 * k + 2) : 0);
+    const size_t off_bytes = 2 * sizeof(u32) * (k + 1) + (use_top ? sizeof(u32) * (2 * k + 2) : 0);
     const size_t up_bytes = sizeof(Inst) * k + off_bytes;
 
     // ---- point workspace
@@ -852,7 +852,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     u32 *lvl_tot = (u32*)P[0], *qlvl_tot = lvl_tot + (size_t)k * LMAX;
     unsigned long long* rec_all = (unsigned long long*)(qlvl_tot + (size_t)k * LMAX);
     Inst* d_inst = (Inst*)(rec_all + k);
-    u32 *d_pt_offs = (u32*)(d_inst + k), *d_chunk_off = d_pt_offs + 2 * (k + 1), *d_prange = d_chunk_off + k + 1,
+    u32 *d_pt_offs = (u32*)(d_inst + k), *d_chunk_off = d_pt_offs + (k + 1), *d_prange = d_chunk_off + k + 1,
         *d_multi = d_prange + k + 1;
     u32* d_pt_tiles = (u32*)P[3];
     u32 *rk0 = (u32*)P[4], *rk1 = (u32*)P[5], *lk = (u32*)P[6], *kalt = (u32*)P[7];
@@ -890,11 +890,10 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         memcpy(hp + lvl_bytes, inst.data(), sizeof(Inst) * k);
         u32* ho = (u32*)(hp + lvl_bytes + sizeof(Inst) * k);
         memcpy(ho, pt_offs.data(), sizeof(u32) * (k + 1));
-        memcpy(ho + (k + 1), q_offs.data(), sizeof(u32) * (k + 1));
-        memcpy(ho + 2 * (k + 1), chunk_off.data(), sizeof(u32) * (k + 1));
+        memcpy(ho + (k + 1), chunk_off.data(), sizeof(u32) * (k + 1));
         if (use_top) {  // (a planned run reuses the tables its measuring run uploaded)
-            memcpy(ho + 3 * (k + 1), prange_off.data(), sizeof(u32) * (k + 1));
-            memcpy(ho + 4 * (k + 1), multi.data(), sizeof(u32) * multi.size());
+            memcpy(ho + 2 * (k + 1), prange_off.data(), sizeof(u32) * (k + 1));
+            memcpy(ho + 3 * (k + 1), multi.data(), sizeof(u32) * multi.size());
         }
         cudaMemcpyAsync(d_inst, hp + lvl_bytes, up_bytes, cudaMemcpyHostToDevice, stream);
         if (!h->no_alloc) h->pin_state = domagg_ctx::PIN_QUEUED;  // (until this call's synchronisation)

@@ -2,11 +2,13 @@
 //
 // This is the sort primitive of the paper (Definition "Sort", Sec. 2.2) as a
 // GPU "onesweep" sort: one histogram pass computes the digit counts of every
-// pass per segment, then every pass is one kernel whose tiles rank their keys
-// locally and find their global output position with a decoupled look-back
-// over the tiles before them.  Segments (problem instances of a batch) are
-// sorted independently: tiles never straddle a segment and the look-back
-// chains stop at the segment's first tile.  Stability (items with equal
+// pass per segment, then every pass is one kernel whose blocks take ranges of
+// whole tiles and rank a tile's keys locally.  A range's global positions come
+// from the histogram (first pass), from a count and a scan of their own (many
+// ranges: k_range_count, k_range_bases) or from a decoupled look-back over the
+// ranges before it.  Segments (problem instances of a batch) are sorted
+// independently: ranges never straddle a segment and the look-back chains stop
+// at the segment's first range.  Stability (items with equal
 // digits keep their order) is what lets the pipeline pre-order points by the
 // last coordinate and then sort records by node key only (Sec. 5).
 #pragma once
