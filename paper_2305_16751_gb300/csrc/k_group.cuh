@@ -94,10 +94,13 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // group of 2^gS ranks is 2^(gS-1) undoubled ranks.  Also writes gbits[s],
 // the bits the group sort sorts: the group id's (b0 - gS) and, for m = 3, the
 // role's.
-// m = 3: a point of a group of c points meets c / 8 pairs, 6e-8 c us at 2.1e6
-// pairs per us, and spares a level's records, b1 / 4 of them at 4e-5 us, for
-// each of the S levels below the group: a width pays while c (over the points)
-// is at most 160 S b1.  (6e5 points, 200 first ranks, S = 1 and 6000 points a
+// m = 3 with records above the groups: a point of a group of c points meets
+// c / 8 pairs, 6e-8 c us at 2.1e6 pairs per us, and spares a level's records,
+// b1 / 4 of them at 4e-5 us, for each of the S levels below the group: a width
+// pays while c (over the points) is at most 160 S b1.  Above it by items a
+// level less also halves the nodes, and the widest stays (2.1e6 points of the
+// empirical CDF, S = 2, 4600 points a group: 2.8 ms, without groups 3.5).
+// (6e5 points, 200 first ranks, S = 1 and 6000 points a
 // group: 748 us without groups, 969 with, second ranks of 8 bits; 1072 and
 // 1230 of 20 bits.  1.9e6 points in 24 instances of 200 ranks, S = 4, 6400
 // points: 2473 us, 2691 at S = 2, of 20 bits; 1856 and 1764 of 5 bits.)
@@ -121,6 +124,18 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
     u32 chosen = 0, G = 0;
     const bool eligible = (M == 2 || M == 3) && rstart && n > 0 && b0 > 0 &&
                           !(I.flags & (FLAG_WAVELET | FLAG_VIRTUAL_LAST));
+    // m = 3: the levels above the groups by items (k_items.cuh), if their nodes
+    // (2^levels - 1 at most) lie within the instance's share of the limit and
+    // the records they replace, half of the second rank's bits for an item,
+    // pay for the items and the nodes' launches (ITEM_MIN_GAIN).  Decided
+    // here, before the records are counted: a call found to hold too many
+    // nodes afterwards would start again (a third of the points on one value,
+    // so without groups, and the others spread: as many nodes as ranks)
+    auto items_gain = [&](u32 levels) -> bool {
+        if (M != 3 || levels == 0u || (1ull << levels) - 1ull > (((u64)n * node_share) >> 32)) return false;
+        return node_min == 0u || (I.b[1] > ITEM_FREE_BITS && levels * (I.b[1] - ITEM_FREE_BITS) >= node_min);
+    };
+    bool by_items = false, decided = false;
     for (int S = eligible ? min(min(max_bits, GROUP_MAX_BITS), (int)b0) : 0; S >= 1; --S) {
         const u32 us = (u32)S - ns;  // undoubled ranks per group: 2^us
         const u32 g_n = (Uu + (1u << us) - 1u) >> us;
@@ -149,13 +164,18 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
             sq += s_sq[w];
         }
         bool ok = ov <= n / 4u && n <= (u64)avg * g_n;
-        if (M == 3 && avg != 0xffffffffu) ok = ok && sq <= (u64)n * (G3_PAIRS_PER_BIT * (u32)S * I.b[1]);
+        if (M == 3 && ok && avg != 0xffffffffu) {
+            if (!decided) by_items = items_gain(b0 - (u32)S);
+            decided = true;
+            ok = by_items || sq <= (u64)n * (G3_PAIRS_PER_BIT * (u32)S * I.b[1]);
+        }
         if (ok && (!chosen || ov == 0u)) chosen = (u32)S;
         // m = 2: on to a narrower width without overflow, as long as the
         // levels above it fit the top tiles
         const bool narrower = M == 2 && top_bits > 0 && S > 1 && b0 - (u32)(S - 1) <= (u32)top_bits;
         if (chosen && (ov == 0u || !narrower)) break;
     }
+    if (M == 3 && !decided) by_items = items_gain(b0);  // no width qualifies: every level
     if (chosen) {
         G = (Uu + (1u << (chosen - ns)) - 1u) >> (chosen - ns);
     }
@@ -191,17 +211,7 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
                 if (lv >= tS) tmask |= 1u << lv;
                 else mask |= 1u << lv;
             }
-        // the levels above the groups by items (k_items.cuh), if their nodes
-        // (2^(b0 - gS) - 1 at most) lie within the instance's share of the
-        // limit; decided here, before the records are counted, since a call
-        // found to hold too many afterwards would start again (a third of the
-        // points on one value, so without groups, and the others spread: as
-        // many nodes as ranks).  And if the records they replace, a level's
-        // item for half of the second rank's bits each, are enough to pay for
-        // the items and the nodes' launches (ITEM_MIN_GAIN)
-        const u32 b1 = I.b[1];
-        if (M == 3 && mask && (1ull << (b0 - chosen)) - 1ull <= (((u64)n * node_share) >> 32) &&
-            (node_min == 0u || (b1 > ITEM_FREE_BITS && (b0 - chosen) * (b1 - ITEM_FREE_BITS) >= node_min))) {
+        if (M == 3 && by_items) {
             tmask = mask;
             mask = 0;
         }

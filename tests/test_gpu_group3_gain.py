@@ -42,3 +42,30 @@ def test_groups_where_their_pairs_pay(n, values0, values1, shared):
         assert t.equal(plan.outs[0], out)
     finally:
         plan.close()
+
+
+def test_groups_stay_where_the_levels_above_go_by_items():
+    """The empirical CDF at 2^20 points: 4600 points a group on average, more
+    than the records of two levels would pay for, but a level less by items
+    halves the nodes."""
+    t = torch()
+    g = t.Generator(device="cuda").manual_seed(10280)
+    X = (t.randn((1 << 20, 3), device="cuda", generator=g) * 256).round() / 256
+    h = domagg.handle(0)
+    domagg.domagg_timing_read(h)
+    domagg.domagg_timing_enable(h, True)
+    try:
+        out = domagg.forward(X, X, None, "count", nonstrict=7)
+        kinds = domagg.domagg_timing_read(h)
+    finally:
+        domagg.domagg_timing_enable(h, False)
+    # the items, from the algorithmic bytes of their two kernels (256 per
+    # 32-point chunk, 12 + 20 per item): a level holds every point once, as
+    # datum or as query; the two levels below the groups hold none
+    items = (kinds["expand"]["bytes"] - 2**21 / 32 * 256) / 32
+    assert 0 < items <= (domagg.stats()["rank_bits"][0] - 2) * 2**20, items / 2**20
+    domagg.domagg_set_tuning(h, "nodes", 0)
+    try:
+        assert t.equal(out, domagg.forward(X, X, None, "count", nonstrict=7))
+    finally:
+        domagg.domagg_set_tuning(h, "nodes", 1)
