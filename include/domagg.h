@@ -224,9 +224,12 @@ typedef struct {
  * sorts, scans and reductions restart at instance boundaries).  `inst` is a
  * host array of k descriptors; coord/weight dtype and op are shared.  Like
  * domagg_forward, the call synchronises `stream` once per group of
- * instances with the same m (to read their record counts) and once more per
+ * instances with the same m (to read their record counts; m = 3: per part of
+ * at most 2^25 points, and for its nodes' sizes) and once more per
  * record chunk when the records of a group do not fit the workspace at once
- * (a chunk holds whole instances); the remaining work is left enqueued. */
+ * (a chunk holds whole instances); small instances go by pairs in one launch
+ * per m, without a synchronisation of their own where others follow.  The
+ * remaining work is left enqueued. */
 domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst,
                            domagg_dtype coord_dtype, domagg_dtype weight_dtype, domagg_op op,
                            void* stream);
@@ -237,8 +240,9 @@ domagg_status domagg_batch(domagg_handle h, int k, const domagg_instance* inst,
  * counterpart (it is the pipeline of domagg_batch, Sec. 4 with Sec. 5, with
  * its host-side layout step moved to the device).
  *
- * domagg_batch_plan runs the batch on `stream` twice (writing the outputs
- * each time) and returns when both runs have finished: the first run
+ * domagg_batch_plan runs the batch on `stream` twice (instances that go by
+ * pairs: once), writing the outputs each time, and returns when the runs have
+ * finished: the first run
  * measures every instance's record counts; the plan then reserves, in a
  * private workspace on `device`, room for (1 + headroom) times those counts
  * (plus 1024) per record chunk and key class (m >= 3: node keys of up to 31
@@ -394,6 +398,9 @@ domagg_status domagg_forward_noalloc(int m, const void* d_coords, int64_t nD, co
  *                    gain, 2: up to 2^25 (never with a capped workspace, in a plan or a
  *                    shard, or with group_bits off its default).  These calls
  *                    synchronise the stream twice more;
+ *   "walk3"          0, 1 or 2 (default 1): for m = 3, the groups of ranks by
+ *                    walks over their levels instead of by pairs; 1: where
+ *                    the coordinates have few distinct values, 2: always;
  *   "rank_windows"   0 .. 64 (default 0: about 48 MB of ranks each): windows
  *                    of destination indices the rank scatter is split into;
  *   "ranges_per_cta" 1 .. 64 (default 4): radix-sort ranges per resident CTA;

@@ -58,7 +58,7 @@ struct Inst {
     u32 b[3];          // binary digits of the ranks: ceil(log2 U)
     u32 rec_off, T;    // records of this instance
     u32 qrec_off, Tq;  // query records (partial slots) of this instance
-    u32 key_bits;      // bits of the node key
+    u32 walk;          // m = 3: the groups by level walks (k_walk3), not by pairs
     u32 flags;         // bit i (i < 3): coordinate i compared non-strictly; FLAG_VIRTUAL_LAST
     // m = 2, 3: rank levels below gS are aggregated per group of 2^gS ranks
     // in shared memory (k_group, k_group3); G groups.  gS = 0: every level

@@ -23,6 +23,7 @@
 #include "k_radix.cuh"
 #include "k_group.cuh"
 #include "k_group3.cuh"
+#include "k_walk3.cuh"
 #include "k_items.cuh"
 #include "k_records.cuh"
 #include "k_top.cuh"
@@ -84,6 +85,7 @@ struct domagg_ctx {
     bool items_live = false;  // between the nodes' stage and the end of its call
     domagg_ctx* sub = nullptr;
     int nodes = 1;
+    int walk3 = 1;  // m = 3: groups by level walks; tuning knob (0: never, 1: by rule, 2: always)
     // on that handle: the point phase's input, ready-made (ranked keys of at
     // most pre_bits bits, by point; the order of the last coordinate)
     u32 *pre_keys = nullptr, *pre_perm = nullptr;
@@ -722,7 +724,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         inst[s].pt_off = (u32)N;
         inst[s].q_off = (u32)NQ;
         for (int i = 0; i < 3; ++i) inst[s].U[i] = inst[s].b[i] = 0;
-        inst[s].T = inst[s].Tq = inst[s].rec_off = inst[s].qrec_off = inst[s].key_bits = 0;
+        inst[s].T = inst[s].Tq = inst[s].rec_off = inst[s].qrec_off = inst[s].walk = 0;
         const u64 n = (u64)inst[s].nD + inst[s].nQ;
         pt_sizes[s] = n;
         N += n;
@@ -823,6 +825,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         P[49] = c.take<u64>(grp ? N : 0);
         P[50] = c.take<u32>(grp ? k : 0);        // group-id bits per instance
         P[51] = c.take<u32>(grp ? k + 1 : 0);    // group slot offsets
+        P[54] = c.take<u32>(grp && M == 3 ? k + 1 : 0);  // of the instances that walk
         // m = 2 top levels: per query F over its range's top levels, per range
         // F of every top-level node (then the carries)
         P[52] = c.take<typename Op::Acc>(use_top ? N : 0);
@@ -864,6 +867,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
     u32* d_sort_tiles = (u32*)P[21];
     u32* chunk_base = (u32*)P[22];
     u32 *rstart = (u32*)P[45], *gkey[2] = {(u32*)P[46], (u32*)P[47]}, *gbits = (u32*)P[50], *gslot = (u32*)P[51];
+    u32* wslot = M == 3 ? (u32*)P[54] : nullptr;
     u64* gval[2] = {(u64*)P[48], (u64*)P[49]};
     typename Op::Acc* topv = (typename Op::Acc*)P[52];
     typename Op::Part* gacc = (typename Op::Part*)P[56];
@@ -1082,8 +1086,9 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                                             govf, M == 3 ? G3_CAP : group_cap(gavg), gavg,
                                             use_groups ? h->group_bits : 0,
                                             use_top ? h->top_bits : 0, items ? (ITEM_MAX_NODES << 32) / N : 0,
-                                            h->nodes == 2 ? 0u : (u32)((ITEM_MIN_GAIN + N - 1) / N), rec_all,
-                                            use_groups && k == 1 ? gslot : nullptr);
+                                            h->nodes == 2 ? 0u : (u32)((ITEM_MIN_GAIN + N - 1) / N), h->walk3,
+                                            (u32)N, (u32)std::max(h->sms, 1), rec_all,
+                                            use_groups && k == 1 ? gslot : nullptr, wslot);
     L.stop();
     // ---- count / offset scan of the flat map, per level
     {
@@ -1323,7 +1328,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
         if (!planned) {
             gb_host.resize(k);
             for (int s = 0; s < k; ++s) {
-                gb_host[s] = inst[s].gS ? inst[s].b[0] - inst[s].gS + (M == 3 ? 1u : 0u) : 0u;  // (m = 3: and the role)
+                gb_host[s] = inst[s].gS ? inst[s].b[0] - inst[s].gS + (M == 3 && !inst[s].walk ? 1u : 0u) : 0u;  // (pairs: and the role)
                 gbits_max = std::max(gbits_max, (int)gb_host[s]);
             }
         } else {  // bound: ranks below 2n (a non-strict first coordinate doubles them)
@@ -1340,7 +1345,7 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
                              gbits, true);
         if (k > 1) {
             L.start(KIND_SMALL, 0.0);
-            k_group_slots<<<1, 1024, 0, stream>>>(d_inst, k, gslot);
+            k_group_slots<<<M == 3 ? 2 : 1, 1024, 0, stream>>>(d_inst, k, gslot, wslot);
             L.stop();
         }
         typedef typename Op::Acc Acc;
@@ -1371,9 +1376,17 @@ domagg_status run(domagg_ctx* h, std::vector<Inst>& inst, bool negate, cudaStrea
             // (data) the weight gathered by position, a partial per query
             L.start(KIND_GROUP, (double)N * (8.0 + 4.0) + (double)(N - NQ) * (WT == 3 ? 0.0 : sizeof(W)) +
                                     (double)NQ * sizeof(Part));
-            k_group3<Op, WT><<<2u * (unsigned)h->sms, PAIR_THREADS, 0, stream>>>(d_inst, k, gslot, rstart, gval[0],
-                                                                                 gval[1], pr1, (const W*)P[18], gacc,
-                                                                                 h->ctl, li);
+            bool by_pairs = planned != nullptr, by_walks = planned != nullptr;  // (a plan's data choose)
+            for (int s = 0; s < k && !planned; ++s) (inst[s].walk ? by_walks : by_pairs) |= inst[s].G > 0;
+            if (by_pairs)
+                k_group3<Op, WT><<<2u * (unsigned)h->sms, PAIR_THREADS, 0, stream>>>(
+                    d_inst, k, gslot, rstart, gval[0], gval[1], pr1, (const W*)P[18], gacc, h->ctl, li);
+            if (by_walks) {
+                constexpr size_t wsm = W3Smem<Acc>::TOTAL;
+                if (!L.frozen) cudaFuncSetAttribute(k_walk3<Op, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm);
+                k_walk3<Op, WT><<<(unsigned)h->sms, W3_THREADS, wsm, stream>>>(
+                    d_inst, k, wslot, rstart, gval[0], gval[1], pr1, (const W*)P[18], gacc, h->ctl, L.lookback_index());
+            }
             L.stop();
         }
     }
@@ -1757,14 +1770,14 @@ bool output_is_input(const std::vector<Inst>* groups, domagg_dtype wt, domagg_op
 
 // Where the line lies: a problem of at most PSTAT_MAX points (its statistics
 // then fit one cluster's shared memory), that is at most 1.5e8 pairs
-// (|D| x |Q|): 63e6 pairs of m = 3 take 30 us, where the pipeline's launches
-// alone take 0.27 ms (m = 2), 0.9 (m = 3), 1.5 (m = 4).  Whole calls,
-// measured: 4096 per side, m = 2, 272 -> 56 us; 12000 x 9001, m = 4,
-// 1519 -> 91 us.  A batch whose such problems hold at most PAIRS_ALL pairs
+// (|D| x |Q|): 63e6 pairs of m = 3 take 36 us.  The pairs would win well above
+// it: calls of 26000 points take 0.28 ms (m = 2), 0.44 (m = 3), 1.67 (m = 4)
+// through the pipeline, launches most of them.  Whole calls, measured: 4096
+// per side, m = 2, 272 -> 48 us; 12000 x 9001, m = 4, 1519 -> 89 us.  A batch whose such problems hold at most PAIRS_ALL pairs
 // together sends them all by pairs (192 problems of 256 to 4096 per side,
 // planned: 1.24 -> 0.24 ms); one with larger instances, which pay for the
 // pipeline's launches, only those of at most PAIRS_EACH pairs: the pairs'
-// throughput (2.5e6 per us for m = 2, 2.1e6 for m = 3) against the pipeline's
+// throughput (2.0e6 per us for m = 2, 1.8e6 for m = 3) against the pipeline's
 // (4000 points per us for m = 2, 1000 for m = 3) meets at about 500 and 2000
 // points per side.
 constexpr u64 PAIRS_ALL[5] = {0, 1ull << 27, 600000000ull, 500000000ull, 2000000000ull};
@@ -2103,6 +2116,9 @@ bool set_tuning(domagg_ctx* h, const std::string& name, int value) {
     } else if (name == "nodes") {
         if (value < 0 || value > 2) return false;
         h->nodes = value;
+    } else if (name == "walk3") {
+        if (value < 0 || value > 2) return false;
+        h->walk3 = value;
     } else if (name == "pairs") {
         if (value < 0 || value > 1) return false;
         h->use_pairs = value != 0;

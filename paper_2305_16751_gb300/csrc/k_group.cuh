@@ -91,9 +91,10 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // per point the call's nodes' path takes (m = 3, in 2^-32; 0: none); node_min:
 // ITEM_MIN_GAIN over the call's points (0: no such limit).  A non-strict
 // first coordinate doubles the ranks (2r for data, 2r+1 for queries), so a
-// group of 2^gS ranks is 2^(gS-1) undoubled ranks.  Also writes gbits[s],
-// the bits the group sort sorts: the group id's (b0 - gS) and, for m = 3, the
-// role's.
+// group of 2^gS ranks is 2^(gS-1) undoubled ranks.  walk_mode: the knob
+// "walk3"; n_total: the call's points.  Also writes gbits[s],
+// the bits the group sort sorts: the group id's (b0 - gS) and, for the pairs of
+// m = 3, the role's.
 // m = 3 with records above the groups: a point of a group of c points meets
 // c / 8 pairs, 6e-8 c us at 2.1e6 pairs per us, and spares a level's records,
 // b1 / 4 of them at 4e-5 us, for each of the S levels below the group: a width
@@ -105,13 +106,33 @@ __device__ __forceinline__ u32 group_slots(u32 shard, u32 nshards, u32 G) {
 // 1230 of 20 bits.  1.9e6 points in 24 instances of 200 ranks, S = 4, 6400
 // points: 2473 us, 2691 at S = 2, of 20 bits; 1856 and 1764 of 5 bits.)
 constexpr u32 G3_PAIRS_PER_BIT = 160;
+// Where level walks (k_walk3) beat the pairs (walk_mode 1): what a point costs,
+// in 1e-8 us, fitted to 216 calls, batches and plans of 4e4 to 2.4e6 points, 3
+// to 4e6 values in the first two coordinates, and the empirical CDF (the route
+// taken lies 0.3 % above the better one on average, 7 % at most; by pairs alone
+// 3.2 % and 36 %).  A
+// walk: its steps (first-rank levels times the bits of a group's second ranks,
+// and a split per first-rank level) and the ranking of the second ranks, one
+// group per SM at a time; pairs: eight times a pair; a level above the groups:
+// its records by their sort's passes, or its item.
+constexpr u32 WALK3_STEP = 300, WALK3_RANK = 200, WALK3_PAIR = 6, WALK3_REC = 500, WALK3_REC_PASS = 250,
+              WALK3_ITEM = 3000, WALK3_ITEM_BIT = 800;
+__device__ __forceinline__ u32 walk3_records(u32 b0, u32 b1, u32 S) {
+    u32 c = 0;
+    for (u32 lv = S; lv < b0; ++lv) {
+        const u32 bits = b0 - 1u - lv + b1;
+        c += b1 * (WALK3_REC + WALK3_REC_PASS * ((bits + 7u) / 8u));
+    }
+    return c;
+}
 constexpr u32 ITEM_FREE_BITS = 6;  // bits of the second rank whose records cost what an item costs
 template <int M>
 __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __restrict__ rstart,
                                                     u32* __restrict__ gbits, unsigned char* __restrict__ govf,
-                                                    u32 cap, u32 avg, int max_bits, int top_bits, u64 node_share, u32 node_min,
+                                                    u32 cap, u32 avg, int max_bits, int top_bits, u64 node_share,
+                                                    u32 node_min, int walk_mode, u32 n_total, u32 sms,
                                                     unsigned long long* __restrict__ rec_all,
-                                                    u32* __restrict__ gslot_off) {
+                                                    u32* __restrict__ gslot_off, u32* __restrict__ wslot_off) {
     __shared__ u32 s_ovf[32];
     __shared__ u64 s_sq[32];
     const int s = blockIdx.x;
@@ -136,6 +157,8 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
         return node_min == 0u || (I.b[1] > ITEM_FREE_BITS && levels * (I.b[1] - ITEM_FREE_BITS) >= node_min);
     };
     bool by_items = false, decided = false;
+    u32 wS = 0;  // m = 3: the widest groups a walk can take
+    u64 wsq = 0, psq = 0;
     for (int S = eligible ? min(min(max_bits, GROUP_MAX_BITS), (int)b0) : 0; S >= 1; --S) {
         const u32 us = (u32)S - ns;  // undoubled ranks per group: 2^us
         const u32 g_n = (Uu + (1u << us) - 1u) >> us;
@@ -169,13 +192,40 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
             decided = true;
             ok = by_items || sq <= (u64)n * (G3_PAIRS_PER_BIT * (u32)S * I.b[1]);
         }
-        if (ok && (!chosen || ov == 0u)) chosen = (u32)S;
+        if (M == 3 && !wS && ov <= n / 4u) {
+            wS = (u32)S;
+            wsq = sq;
+        }
+        if (ok && (!chosen || ov == 0u)) {
+            chosen = (u32)S;
+            psq = sq;
+        }
         // m = 2: on to a narrower width without overflow, as long as the
         // levels above it fit the top tiles
         const bool narrower = M == 2 && top_bits > 0 && S > 1 && b0 - (u32)(S - 1) <= (u32)top_bits;
         if (chosen && (ov == 0u || !narrower)) break;
     }
-    if (M == 3 && !decided) by_items = items_gain(b0);  // no width qualifies: every level
+    bool walk = false;
+    if (M == 3) {
+        if (!decided) by_items = items_gain(b0);  // no width qualifies: every level
+        if (wS && walk_mode == 1 && !(by_items && node_min == 0u)) {  // (nodes = 2: always by items)
+            const u32 b1 = I.b[1], cw = max(1u, (u32)(wsq / n));
+            const u32 lb = min(b1, 32u - __clz(cw));  // bits of a group's second ranks
+            // groups in the call, its instances taken as alike
+            const u32 g = max(1u, n_total / cw), waves = (g + sms - 1u) / sms;
+            const u64 steps = (u64)(wS * lb + wS) * WALK3_STEP + b1 * WALK3_RANK;
+            const u64 walks = steps * waves * sms / g + walk3_records(b0, b1, wS);
+            const u64 pairs = (psq / n) * WALK3_PAIR +
+                              (by_items ? (u64)(b0 - chosen) * (WALK3_ITEM + WALK3_ITEM_BIT * b1) + 10000000000ull / n_total
+                                        : walk3_records(b0, b1, chosen));
+            walk = walks * 11u < pairs * 10u;
+            if (walk) by_items = false;
+        } else if (wS && walk_mode == 2) {
+            walk = true;
+            by_items = items_gain(b0 - wS);
+        }
+        if (walk) chosen = wS;
+    }
     if (chosen) {
         G = (Uu + (1u << (chosen - ns)) - 1u) >> (chosen - ns);
     }
@@ -194,11 +244,17 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
         I.gS = chosen;
         I.G = chosen ? G : 0u;
         rec_all[s] = 0ull;  // (the count scan adds up)
+        I.walk = walk ? 1u : 0u;
         if (gslot_off) {    // a single instance: its slots (else k_group_slots)
+            const u32 slots = chosen ? group_slots(I.shard, I.nshards, G) : 0u;
             gslot_off[0] = 0u;
-            gslot_off[1] = chosen ? group_slots(I.shard, I.nshards, G) : 0u;
+            gslot_off[1] = walk ? 0u : slots;
+            if (wslot_off) {
+                wslot_off[0] = 0u;
+                wslot_off[1] = walk ? slots : 0u;
+            }
         }
-        if (gbits) gbits[s] = chosen ? b0 - chosen + (M == 3 ? 1u : 0u) : 0u;
+        if (gbits) gbits[s] = chosen ? b0 - chosen + (M == 3 && !walk ? 1u : 0u) : 0u;
         // the levels >= gS of this shard: from tS up per tile (k_top), below
         // tS through the records in HBM
         const u32 nlev = M == 1 ? 1u : b0;
@@ -223,9 +279,11 @@ __global__ __launch_bounds__(1024) void k_group_plan(Inst* inst, const u32* __re
 }
 
 // Work list of k_group: slot offsets of the instances' groups (exclusive
-// scan of G over the instances that use groups).  One block.
-static __global__ __launch_bounds__(1024) void k_group_slots(const Inst* __restrict__ inst, int k,
-                                                            u32* __restrict__ gslot_off) {
+// scan of G over the instances that use groups).  With wslot_off, those of the
+// instances that walk go there (m = 3: k_walk3's list).  One block per list.
+static __global__ __launch_bounds__(1024) void k_group_slots(const Inst* __restrict__ inst, int k, u32* pslot_off,
+                                                            u32* wslot_off) {
+    u32* gslot_off = blockIdx.x ? wslot_off : pslot_off;
     __shared__ u32 carry;
     __shared__ u32 warp_sum[32];
     if (threadIdx.x == 0) carry = 0;
@@ -234,7 +292,8 @@ static __global__ __launch_bounds__(1024) void k_group_slots(const Inst* __restr
     for (int base = 0; base < k; base += blockDim.x) {
         const int s = base + threadIdx.x;
         u32 v = 0;
-        if (s < k && inst[s].gS) v = group_slots(inst[s].shard, inst[s].nshards, inst[s].G);
+        if (s < k && inst[s].gS && (!wslot_off || inst[s].walk == blockIdx.x))
+            v = group_slots(inst[s].shard, inst[s].nshards, inst[s].G);
         u32 inc = v;
         for (int o = 1; o < 32; o <<= 1) {
             const u32 x = __shfl_up_sync(0xffffffffu, inc, o);

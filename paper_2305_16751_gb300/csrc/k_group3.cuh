@@ -47,7 +47,8 @@ __host__ __device__ constexpr u32 g3_avg(u64 N, bool tight, bool items) {
     return c >= 7168u ? 7168u : (c <= 1024u ? 1024u : (u32)c);
 }
 
-// The deep levels of every m = 3 group (see the file comment).  Persistent
+// The deep levels of every group of the instances that go by pairs (see the
+// file comment).  Persistent
 // blocks take (query tile, group) pairs from a counter, a group's last tiles
 // (the most data before them) first.  Inputs: the group-sorted points gv (per
 // instance in buffer gv0 or gv1, by the parity of the group sort's passes):

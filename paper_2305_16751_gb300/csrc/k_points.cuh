@@ -495,7 +495,8 @@ __global__ __launch_bounds__(256) void k_count_scan(
             // for m = 3, its position x)
             if ((M == 2 || M == 3) && gkey && I.gS) {
                 const u32 pv = (q || WT == 1 || M == 3) ? x : wbits;
-                gkey[x] = M == 3 ? ((a >> I.gS) << 1) | (q ? 1u : 0u) : a >> I.gS;  // (m = 3: data first)
+                // (m = 3 by pairs: data first)
+                gkey[x] = M == 3 && !I.walk ? ((a >> I.gS) << 1) | (q ? 1u : 0u) : a >> I.gS;
                 gval[x] = ((u64)(q ? (a | QUERY_BIT) : a) << 32) | (u64)pv;
             }
         }
