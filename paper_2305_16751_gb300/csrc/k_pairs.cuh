@@ -6,8 +6,9 @@
 // definition out(q) = F{ w(d) : d_i < q_i for all i } evaluated over all
 // (d, q) pairs needs no order, no rank and no record: m compares, one select
 // and one F per pair on every multiprocessor, 10 instructions for m = 2 with
-// the float-float sum, so 4096 x 4096 pairs take about 5 us and the call is
-// one launch (plus the flat-map statistics beside it, k_pair_stats).
+// the float-float sum (2.0e6 pairs per us at 8000 x 8000; 4096 x 4096 take 16 us
+// beside the statistics), and the call is one launch plus the flat-map
+// statistics beside it (k_pair_stats).
 #pragma once
 #include "dev_common.cuh"
 #include "k_points.cuh"
